@@ -11,6 +11,8 @@
 #include "../../include/spd.h"
 #include "spd_kernel.cuh"
 #include "spd_prefill.cuh"
+#include "spd_gemm.cuh"
+#include "spd_attn.cuh"
 #include "spd_warp.cuh"
 #include "spd_tree.cuh"
 #include "spd_batch.cuh"
@@ -74,10 +76,10 @@ struct spd_ctx {
   // scratch of the tensor-core prefill, grown on demand
   struct {
     size_t cap_rows = 0;
-    __nv_bfloat16 *h_hi = nullptr, *h_lo = nullptr, *q_hi = nullptr, *q_lo = nullptr, *vT = nullptr;
-    __nv_bfloat16 *p_hi = nullptr, *p_lo = nullptr;
+    __nv_bfloat16 *h_hi = nullptr, *h_lo = nullptr, *q_hi = nullptr, *q_lo = nullptr;
     __nv_bfloat16 *g_hi = nullptr, *g_lo = nullptr;   // silu(gate) * up [rows][d_ffn]
-    float *wide = nullptr, *S = nullptr;
+    float* wide = nullptr;                            // projection results, K slice by K slice
+    size_t cap_wide = 0;
   } pf;
   // scratch of spd_image_adapter, grown on demand
   struct {
@@ -624,83 +626,116 @@ EncodeTiledFn encode_tiled_fn() {
   return fn;
 }
 
-// bf16 operand view [batch][rows][inner] with byte strides; box = 64 inner x 128 rows x 1.
-spd_status make_map(spd_ctx* ctx, CUtensorMap* m, const void* ptr, int inner, int rows, int batch, size_t row_stride,
-                    size_t batch_stride, int box_rows = TC_BM) {
+// bf16 matrix [rows][inner], dense rows; box = 64 columns x box_rows.
+spd_status make_map(spd_ctx* ctx, CUtensorMap* m, const void* ptr, int inner, int rows, int box_rows) {
   EncodeTiledFn fn = encode_tiled_fn();
   if (!fn) return fail(ctx, SPD_ECUDA, "cuTensorMapEncodeTiled not available");
-  const cuuint64_t dims[3] = {(cuuint64_t)inner, (cuuint64_t)rows, (cuuint64_t)batch};
-  const cuuint64_t strides[2] = {(cuuint64_t)row_stride, (cuuint64_t)batch_stride};
+  const cuuint64_t dims[3] = {(cuuint64_t)inner, (cuuint64_t)rows, 1};
+  const cuuint64_t strides[2] = {(cuuint64_t)inner * 2, (cuuint64_t)inner * 2 * rows};
   const cuuint32_t box[3] = {(cuuint32_t)TC_BK, (cuuint32_t)box_rows, 1};
   const cuuint32_t estr[3] = {1, 1, 1};
   const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(ctx, SPD_ECUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
   return SPD_OK;
 }
 
-struct Operand { const void* ptr; int inner, rows, batch; size_t row_stride, batch_stride; };
+// A launch that may start while its predecessor in the stream still runs (the kernel calls pdl_wait).
+template <class... KA, class... A>
+cudaError_t launch_dependent(void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, KA(args)...);
+}
 
-// stream_ksplit = 0: the prefill form (3 stages, two CTAs per SM).  > 0: few rows against a large
-// weight matrix -- 6 stages, one CTA per SM, and the K loop cut into that many slices so that
-// enough CTAs stream; the slices' partial products go to `ws` and are summed in slice order.
-// `wide`: weight-tile rows of the streaming form (0 or 128, 160, 256): the wider, the fewer activation bytes
-// re-read per weight byte.
-spd_status tc_gemm(spd_ctx* ctx, const Operand& a_hi, const Operand& a_lo, const Operand& b, TcArgs args,
-                   bool gelu = false, int stream_ksplit = 0, float* ws = nullptr, int wide = 0,
-                   bool leave_slices = false) {
-  CUtensorMap ma, ml, mb;
-  spd_status s;
-  if ((s = make_map(ctx, &ma, a_hi.ptr, a_hi.inner, a_hi.rows, a_hi.batch, a_hi.row_stride, a_hi.batch_stride))) return s;
-  if ((s = make_map(ctx, &ml, a_lo.ptr, a_lo.inner, a_lo.rows, a_lo.batch, a_lo.row_stride, a_lo.batch_stride))) return s;
-  if ((s = make_map(ctx, &mb, b.ptr, b.inner, b.rows, b.batch, b.row_stride, b.batch_stride,
-                    stream_ksplit > 0 && wide > 0 ? wide : TC_BN))) return s;
-  static bool attr_set[MAX_DEV];
-  if (ctx->device < 0 || ctx->device >= MAX_DEV) return fail(ctx, SPD_ECUDA, "device index out of range");
-  if (!attr_set[ctx->device]) {
-    CU(cudaFuncSetAttribute((const void*)tc_gemm_kernel<false, TC_STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BYTES));
-    CU(cudaFuncSetAttribute((const void*)tc_gemm_kernel<true, TC_STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BYTES));
-    CU(cudaFuncSetAttribute((const void*)tc_gemm_kernel<false, TC_STAGES_STREAM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            tc_smem_bytes(TC_STAGES_STREAM)));
-    CU(cudaFuncSetAttribute((const void*)tc_gemm_kernel<false, TC_STAGES_WIDE, TC_BN_WIDE>,
-                            cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem_bytes(TC_STAGES_WIDE, TC_BN_WIDE)));
-    CU(cudaFuncSetAttribute((const void*)tc_gemm_kernel<false, TC_STAGES_MID, TC_BN_MID>,
-                            cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem_bytes(TC_STAGES_MID, TC_BN_MID)));
-    attr_set[ctx->device] = true;
-  }
-  args.split = 1;
-  args.err = &ctx->st->err;
-  args.ksplit = 1;
-  if (stream_ksplit > 0) {
-    if (gelu || a_hi.batch != 1 || args.mode == TC_OUT_SPLIT || (args.mode == TC_OUT_SWIGLU && stream_ksplit > 1))
-      return fail(ctx, SPD_EINVAL, "streaming GEMM: fp32 output, or the SwiGLU epilogue on an unsliced K");
-    const int mode = args.mode;
-    float* dest = args.out_f32;
-    const long long ldo = args.ldo;
-    if (stream_ksplit > 1) {
-      if (!ws || ldo != args.N) return fail(ctx, SPD_EINVAL, "split GEMM needs a workspace and a dense output");
-      args.ksplit = stream_ksplit; args.out_f32 = ws; args.mode = TC_OUT_F32;
+// How a dense linear map is cut up: CTA pairs or single CTAs, rows per activation tile, K slices.
+struct UgPlan { int cg, bn, slices; };
+
+// The plan with the smallest modelled time.  Per 64-wide K block a unit needs the longest of: its MMAs
+// (8 instructions of bn / 2 cycles at the ~1.4 GHz the power limit leaves a dense tensor loop), its
+// share of the L2 -> SM traffic (weights 16 KB + activations 256 * bn bytes per CTA, halved by pairing,
+// at 85 KB/us per SM: what the 128-row tiles of a 640-row gate/up projection reached) and, for few
+// rows, HBM (6.2 GB/ms over all CTAs).  A unit does `rounds` items, each with ~1.5 us of pipeline fill
+// and epilogue; every further slice is written and read once more.  The model orders the measured
+// cases right: 640 rows x N 12288 / 22016 / 4096, K 4096: bn 160 95 / 159 / 34 us, 128 100 / 162 / 47,
+// 224 94 / 172 / 44; 96 rows: QKV 3 slices of pairs 28, of single CTAs 30, 2 slices 32.
+UgPlan ug_plan(int n_sm, int R, int N, int K, int max_slices) {
+  UgPlan best{1, 16, 1};
+  double best_t = 1e30;
+  const int kb = (K + TC_BK - 1) / TC_BK;
+  for (int cg = 1; cg <= 2; ++cg) {
+    const int step = cg == 2 ? 32 : 16, units = n_sm / cg, wt = (N + 128 * cg - 1) / (128 * cg);
+    int last_bn = 0;
+    for (int want = (R + UG_BN_MAX - 1) / UG_BN_MAX, i = 0; i < 6; ++i, ++want) {
+      const int bn = ((R + want - 1) / want + step - 1) / step * step;
+      if (bn == last_bn) continue;
+      last_bn = bn;
+      const int n_at = (R + bn - 1) / bn;
+      const long long tiles = (long long)wt * n_at;
+      for (int s = 1; s <= max_slices && s <= kb; ++s) {
+        const long long items = tiles * s, rounds = (items + units - 1) / units;
+        const double ctas = (double)(items < units ? items : units) * cg;
+        const double mma = bn * 4 / 1400.0, l2 = (16384 + 256.0 * bn / cg) / 85e3, hbm = ctas * 16384 / n_at / 6.2e6;
+        double per = mma > l2 ? mma : l2;
+        if (hbm > per) per = hbm;
+        const double t = rounds * (((kb + s - 1) / s) * per + 1.5) + (cg == 2 ? 0.5 : 0.0) + (s - 1) * (double)R * N * 8 / 4e6;
+        if (t < best_t) { best_t = t; best = UgPlan{cg, bn, s}; }
+      }
     }
-    if (wide != 0 && wide != TC_BN && wide != TC_BN_MID && wide != TC_BN_WIDE) return fail(ctx, SPD_EINVAL, "streaming GEMM: tile width");
-    const int bn = wide > 0 ? wide : TC_BN;
-    dim3 grid((args.N + bn - 1) / bn, (args.M + TC_BM - 1) / TC_BM, stream_ksplit);
-    if (bn == TC_BN_WIDE)
-      tc_gemm_kernel<false, TC_STAGES_WIDE, TC_BN_WIDE><<<grid, 128, tc_smem_bytes(TC_STAGES_WIDE, TC_BN_WIDE), ctx->stream>>>(ma, ml, mb, args);
-    else if (bn == TC_BN_MID)
-      tc_gemm_kernel<false, TC_STAGES_MID, TC_BN_MID><<<grid, 128, tc_smem_bytes(TC_STAGES_MID, TC_BN_MID), ctx->stream>>>(ma, ml, mb, args);
-    else
-      tc_gemm_kernel<false, TC_STAGES_STREAM><<<grid, 128, tc_smem_bytes(TC_STAGES_STREAM), ctx->stream>>>(ma, ml, mb, args);
-    if (stream_ksplit > 1 && !leave_slices)   // (leave_slices: the caller's next kernel adds them up)
-      tc_reduce_kernel<<<148, 256, 0, ctx->stream>>>(ws, stream_ksplit, (size_t)args.M * args.N, dest, mode == TC_OUT_F32_ADD);
-    CU(cudaGetLastError());
-    return SPD_OK;
   }
-  dim3 grid((args.N + TC_BN - 1) / TC_BN, (args.M + TC_BM - 1) / TC_BM, a_hi.batch);
-  if (gelu) tc_gemm_kernel<true, TC_STAGES><<<grid, 128, TC_SMEM_BYTES, ctx->stream>>>(ma, ml, mb, args);
-  else tc_gemm_kernel<false, TC_STAGES><<<grid, 128, TC_SMEM_BYTES, ctx->stream>>>(ma, ml, mb, args);
-  CU(cudaGetLastError());
+  return best;
+}
+
+template <int CG, int EPI>
+spd_status ug_launch(spd_ctx* ctx, const CUtensorMap& mw, const CUtensorMap& mh, const CUtensorMap& ml, const UgArgs& a) {
+  static bool attr[MAX_DEV];
+  if (!attr[ctx->device]) {
+    CU(cudaFuncSetAttribute((const void*)umma_gemm_kernel<CG, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, UG_SMEM));
+    attr[ctx->device] = true;
+  }
+  const long long items = (long long)a.tiles * a.slices;
+  const int units = (int)(items < ctx->n_sm / CG ? items : ctx->n_sm / CG);
+  CU(launch_dependent(umma_gemm_kernel<CG, EPI>, dim3(units * CG), dim3(UG_THREADS), UG_SMEM, ctx->stream, mw, mh, ml, a));
   return SPD_OK;
+}
+
+// Y[R][N] = X[R][K] W[N][K]^T, X as bf16 hi + lo, dense rows (K a multiple of 8).  out_f32 receives
+// `slices_out` partial products [slices][R][N] (at most max_slices; 1 where only a whole sum is wanted).
+spd_status ug_gemm(spd_ctx* ctx, const __nv_bfloat16* x_hi, const __nv_bfloat16* x_lo, int R, int K, const void* w, int N,
+                   int epi, float* out_f32, __nv_bfloat16* out_hi, __nv_bfloat16* out_lo, long long ldo, int max_slices = 1,
+                   int* slices_out = nullptr) {
+  if (ctx->device < 0 || ctx->device >= MAX_DEV) return fail(ctx, SPD_ECUDA, "device index out of range");
+  const UgPlan p = ug_plan(ctx->n_sm, R, N, K, max_slices);
+  UgArgs a{};
+  a.N = N; a.R = R; a.K = K;
+  a.bn = p.bn;
+  a.n_at = (R + p.bn - 1) / p.bn;
+  a.kb = (K + TC_BK - 1) / TC_BK;
+  a.tiles = (N + 128 * p.cg - 1) / (128 * p.cg) * a.n_at;
+  a.slices = p.slices;
+  a.stages = UG_RING / (UG_A_BYTES + 2 * (p.bn / p.cg) * TC_BK * 2);
+  if (a.stages > UG_STAGES_MAX) a.stages = UG_STAGES_MAX;
+  a.ldo = ldo; a.out_f32 = out_f32; a.out_hi = out_hi; a.out_lo = out_lo;
+  a.err = &ctx->st->err;
+  if (slices_out) *slices_out = p.slices;
+  CUtensorMap mw, mh, ml;
+  spd_status s;
+  if ((s = make_map(ctx, &mw, w, K, N, 128))) return s;
+  if ((s = make_map(ctx, &mh, x_hi, K, R, p.bn / p.cg))) return s;
+  if ((s = make_map(ctx, &ml, x_lo, K, R, p.bn / p.cg))) return s;
+  if (p.cg == 2) {
+    if (epi == UG_F32) return ug_launch<2, UG_F32>(ctx, mw, mh, ml, a);
+    if (epi == UG_GELU) return ug_launch<2, UG_GELU>(ctx, mw, mh, ml, a);
+    return ug_launch<2, UG_SWIGLU>(ctx, mw, mh, ml, a);
+  }
+  if (epi == UG_F32) return ug_launch<1, UG_F32>(ctx, mw, mh, ml, a);
+  if (epi == UG_GELU) return ug_launch<1, UG_GELU>(ctx, mw, mh, ml, a);
+  return ug_launch<1, UG_SWIGLU>(ctx, mw, mh, ml, a);
 }
 
 // Embedding rows of n token ids.  An id outside [0, V) (possible when the ids live in device
@@ -718,78 +753,86 @@ __global__ void gather_rows_kernel(const int* ids, const float* table, float* ou
   }
 }
 
+// Most K slices of a projection whose reader adds them up, and the rows up to which that is offered
+// (their partial products then fit the widest activation buffer).
+constexpr int UG_SLICES_MAX = 8;
+
 spd_status prefill_scratch(spd_ctx* ctx, int R) {
   if ((size_t)R <= ctx->pf.cap_rows) return SPD_OK;
   const spd_model_cfg &t = ctx->cfg.target, &d = ctx->cfg.draft;
   const size_t dm = t.d_model > d.d_model ? t.d_model : d.d_model;
   const size_t fm = t.d_ffn > d.d_ffn ? t.d_ffn : d.d_ffn;
-  const size_t hm = t.n_heads > d.n_heads ? t.n_heads : d.n_heads;
   const size_t ad = ctx->cfg.draft_adapter_in;
   size_t kin = dm > fm ? dm : fm;
   if (ad > kin) kin = ad;
-  const size_t wide = 3 * dm > 2 * fm ? 3 * dm : 2 * fm;
   const size_t rp = ((size_t)R + 63) / 64 * 64;
+  size_t wide = rp * (3 * dm > ad ? 3 * dm : ad);
+  if (wide < (size_t)UG_SLICES_MAX * BATCH_ROWS_MAX * 3 * dm) wide = (size_t)UG_SLICES_MAX * BATCH_ROWS_MAX * 3 * dm;
   spd_status s;   // earlier buffers stay in the context's allocation list until spd_destroy
   if ((s = dalloc(ctx, &ctx->pf.h_hi, rp * kin))) return s;
   if ((s = dalloc(ctx, &ctx->pf.h_lo, rp * kin))) return s;
   if ((s = dalloc(ctx, &ctx->pf.q_hi, rp * dm))) return s;
   if ((s = dalloc(ctx, &ctx->pf.q_lo, rp * dm))) return s;
-  if ((s = dalloc(ctx, &ctx->pf.vT, dm * rp))) return s;
-  if ((s = dalloc(ctx, &ctx->pf.wide, rp * wide))) return s;
-  if ((s = dalloc(ctx, &ctx->pf.S, hm * rp * rp))) return s;
-  if ((s = dalloc(ctx, &ctx->pf.p_hi, hm * rp * rp))) return s;
-  if ((s = dalloc(ctx, &ctx->pf.p_lo, hm * rp * rp))) return s;
+  if ((s = dalloc(ctx, &ctx->pf.wide, wide))) return s;
   if ((s = dalloc(ctx, &ctx->pf.g_hi, rp * fm))) return s;
   if ((s = dalloc(ctx, &ctx->pf.g_lo, rp * fm))) return s;
+  ctx->pf.cap_wide = wide;
   ctx->pf.cap_rows = rp;
   return SPD_OK;
 }
 
+// K slices that fit the activation buffer for an [R][N] result.
+int slices_that_fit(const spd_ctx* ctx, int R, int N) {
+  const size_t n = ctx->pf.cap_wide / ((size_t)R * N);
+  return n < 1 ? 1 : (n < UG_SLICES_MAX ? (int)n : UG_SLICES_MAX);
+}
+
+template <int DH>
+spd_status launch_prefill_attn(spd_ctx* ctx, const __nv_bfloat16* kc, const __nv_bfloat16* vc, int R, int H, float scale) {
+  static bool attr[MAX_DEV];
+  if (!attr[ctx->device]) {
+    CU(cudaFuncSetAttribute((const void*)prefill_attn_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, pa_smem(DH)));
+    attr[ctx->device] = true;
+  }
+  auto& pf = ctx->pf;
+  CU(launch_dependent(prefill_attn_kernel<DH>, dim3(H * ((R + PA_ROWS - 1) / PA_ROWS)), dim3(PA_THREADS), pa_smem(DH),
+                      ctx->stream, pf.q_hi, pf.q_lo, kc, vc, R, H, ctx->cfg.max_seq, scale, pf.h_hi, pf.h_lo));
+  return SPD_OK;
+}
+
 // Dense forward of rows X [R][d] (fp32, device; positions 0..R-1) through every layer of a
-// bf16 model: fills the KV cache rows 0..R-1 and leaves the final residual stream in X.
+// bf16 model: fills the KV cache rows 0..R-1 and leaves the final residual stream in X.  Seven launches
+// a layer; a projection whose reader can add K slices up is sliced where that fills the device.
 spd_status prefill_tc(spd_ctx* ctx, ModelHost& mh, float* X, int R) {
   const int d = mh.cfg.d_model, f = mh.cfg.d_ffn, H = mh.cfg.n_heads, dh = d / H, L = mh.cfg.n_layers;
-  const int rp = (R + 63) / 64 * 64;
   spd_status s;
   if ((s = prefill_scratch(ctx, R))) return s;
   auto& pf = ctx->pf;
   cudaStream_t cs = ctx->stream;
-  CU(cudaMemsetAsync(pf.vT, 0, (size_t)d * rp * 2, cs));
-  const size_t max_seq = ctx->cfg.max_seq;
+  const size_t max_seq = ctx->cfg.max_seq, xs = (size_t)R * d;
+  const int rope_blocks = (R * (d >> 3) + 255) / 256;
+  CU(launch_dependent(resid_rms_split_kernel, dim3(R), dim3(256), 0, cs, X, pf.wide, 0, xs, mh.rm[0].attn_norm, mh.cfg.rms_eps, d,
+                      pf.h_hi, pf.h_lo));
   for (int l = 0; l < L; ++l) {
     const ModelHost::RowMajor& w = mh.rm[l];
     __nv_bfloat16* kc = static_cast<__nv_bfloat16*>(mh.md.kcache) + (size_t)l * max_seq * d;
     __nv_bfloat16* vc = static_cast<__nv_bfloat16*>(mh.md.vcache) + (size_t)l * max_seq * d;
-    TcArgs a{};
-    // attention block
-    rms_split_kernel<<<R, 256, 0, cs>>>(X, w.attn_norm, mh.cfg.rms_eps, d, pf.h_hi, pf.h_lo);
-    a = TcArgs{}; a.M = R; a.N = 3 * d; a.K = d; a.mode = TC_OUT_F32; a.alpha = 1.f; a.out_f32 = pf.wide; a.ldo = 3 * d;
-    if ((s = tc_gemm(ctx, {pf.h_hi, d, R, 1, (size_t)d * 2, (size_t)R * d * 2}, {pf.h_lo, d, R, 1, (size_t)d * 2, (size_t)R * d * 2},
-                     {w.wqkv, d, 3 * d, 1, (size_t)d * 2, (size_t)3 * d * d * 2}, a))) return s;
-    rope_kv_kernel<<<592, 256, 0, cs>>>(pf.wide, R, d, dh, 0, mh.md.rope_cos, mh.md.rope_sin, pf.q_hi, pf.q_lo, kc, vc,
-                                        pf.vT, rp, (int)max_seq);
-    a = TcArgs{}; a.M = R; a.N = R; a.K = dh; a.mode = TC_OUT_F32; a.alpha = mh.md.scale; a.out_f32 = pf.S; a.ldo = rp;
-    a.out_batch = (long long)R * rp;
-    if ((s = tc_gemm(ctx, {pf.q_hi, dh, R, H, (size_t)d * 2, (size_t)dh * 2}, {pf.q_lo, dh, R, H, (size_t)d * 2, (size_t)dh * 2},
-                     {kc, dh, R, H, (size_t)dh * 2, max_seq * dh * 2}, a))) return s;   // a head's cached rows are contiguous
-    softmax_causal_split_kernel<<<H * R, 256, 0, cs>>>(pf.S, R, rp, pf.p_hi, pf.p_lo);
-    a = TcArgs{}; a.M = R; a.N = dh; a.K = rp; a.mode = TC_OUT_SPLIT; a.alpha = 1.f; a.out_hi = pf.h_hi; a.out_lo = pf.h_lo;
-    a.ldo = d; a.out_batch = dh;
-    if ((s = tc_gemm(ctx, {pf.p_hi, rp, R, H, (size_t)rp * 2, (size_t)R * rp * 2}, {pf.p_lo, rp, R, H, (size_t)rp * 2, (size_t)R * rp * 2},
-                     {pf.vT, rp, dh, H, (size_t)rp * 2, (size_t)dh * rp * 2}, a))) return s;
-    a = TcArgs{}; a.M = R; a.N = d; a.K = d; a.mode = TC_OUT_F32_ADD; a.alpha = 1.f; a.out_f32 = X; a.ldo = d;
-    if ((s = tc_gemm(ctx, {pf.h_hi, d, R, 1, (size_t)d * 2, (size_t)R * d * 2}, {pf.h_lo, d, R, 1, (size_t)d * 2, (size_t)R * d * 2},
-                     {w.wo, d, d, 1, (size_t)d * 2, (size_t)d * d * 2}, a))) return s;
-    // feed-forward block
-    rms_split_kernel<<<R, 256, 0, cs>>>(X, w.ffn_norm, mh.cfg.rms_eps, d, pf.h_hi, pf.h_lo);
+    int sl = 1;
+    if ((s = ug_gemm(ctx, pf.h_hi, pf.h_lo, R, d, w.wqkv, 3 * d, UG_F32, pf.wide, nullptr, nullptr, 3 * d,
+                     slices_that_fit(ctx, R, 3 * d), &sl))) return s;
+    CU(launch_dependent(rope_kv_kernel, dim3(rope_blocks), dim3(256), 0, cs, pf.wide, sl, R, d, dh, mh.md.rope_cos, mh.md.rope_sin,
+                        pf.q_hi, pf.q_lo, kc, vc, (int)max_seq));
+    if ((s = dh == 128 ? launch_prefill_attn<128>(ctx, kc, vc, R, H, mh.md.scale) : launch_prefill_attn<64>(ctx, kc, vc, R, H, mh.md.scale)))
+      return s;
+    if ((s = ug_gemm(ctx, pf.h_hi, pf.h_lo, R, d, w.wo, d, UG_F32, pf.wide, nullptr, nullptr, d, slices_that_fit(ctx, R, d), &sl))) return s;
+    CU(launch_dependent(resid_rms_split_kernel, dim3(R), dim3(256), 0, cs, X, pf.wide, sl, xs, w.ffn_norm, mh.cfg.rms_eps, d, pf.h_hi,
+                        pf.h_lo));
     // gate/up with SwiGLU in the epilogue (interleaved gate/up rows): hi/lo [R][f] straight out of the GEMM
-    a = TcArgs{}; a.M = R; a.N = 2 * f; a.K = d; a.mode = TC_OUT_SWIGLU; a.alpha = 1.f; a.out_hi = pf.g_hi; a.out_lo = pf.g_lo; a.ldo = f;
-    if ((s = tc_gemm(ctx, {pf.h_hi, d, R, 1, (size_t)d * 2, (size_t)R * d * 2}, {pf.h_lo, d, R, 1, (size_t)d * 2, (size_t)R * d * 2},
-                     {w.wgu, d, 2 * f, 1, (size_t)d * 2, (size_t)2 * f * d * 2}, a))) return s;
-    a = TcArgs{}; a.M = R; a.N = d; a.K = f; a.mode = TC_OUT_F32_ADD; a.alpha = 1.f; a.out_f32 = X; a.ldo = d;
-    if ((s = tc_gemm(ctx, {pf.g_hi, f, R, 1, (size_t)f * 2, (size_t)R * f * 2}, {pf.g_lo, f, R, 1, (size_t)f * 2, (size_t)R * f * 2},
-                     {w.wd, f, d, 1, (size_t)f * 2, (size_t)d * f * 2}, a))) return s;
-    CU(cudaGetLastError());
+    if ((s = ug_gemm(ctx, pf.h_hi, pf.h_lo, R, d, w.wgu, 2 * f, UG_SWIGLU, nullptr, pf.g_hi, pf.g_lo, f))) return s;
+    if ((s = ug_gemm(ctx, pf.g_hi, pf.g_lo, R, f, w.wd, d, UG_F32, pf.wide, nullptr, nullptr, d, slices_that_fit(ctx, R, d), &sl))) return s;
+    // the norm in front of the next layer rides on the residual update
+    CU(launch_dependent(resid_rms_split_kernel, dim3(R), dim3(256), 0, cs, X, pf.wide, sl, xs,
+                        l + 1 < L ? mh.rm[l + 1].attn_norm : mh.md.final_norm, mh.cfg.rms_eps, d, pf.h_hi, pf.h_lo));
   }
   return SPD_OK;
 }
@@ -1026,11 +1069,9 @@ spd_status spd_prefill(spd_ctx* ctx, const float* image_embeds, int m, const flo
       dm.pos_base = m;
     } else if (ad > 0) {   // draft rows [H W_a^T ; embed(prompt)]
       CU(cudaMemcpyAsync(ctx->pf.wide, draft_image_feats, (size_t)m * ad * sizeof(float), cudaMemcpyDefault, ctx->stream));
-      split_rows_kernel<<<592, 256, 0, ctx->stream>>>(ctx->pf.wide, ctx->pf.h_hi, ctx->pf.h_lo, (size_t)m * ad);
-      TcArgs a{}; a.M = m; a.N = dd; a.K = ad; a.mode = TC_OUT_F32; a.alpha = 1.f; a.out_f32 = X; a.ldo = dd;
-      if ((s = tc_gemm(ctx, {ctx->pf.h_hi, ad, m, 1, (size_t)ad * 2, (size_t)m * ad * 2},
-                       {ctx->pf.h_lo, ad, m, 1, (size_t)ad * 2, (size_t)m * ad * 2},
-                       {dm.adapter_rm, ad, dd, 1, (size_t)ad * 2, (size_t)dd * ad * 2}, a))) return s;
+      CU(launch_dependent(split_rows_kernel, dim3(592), dim3(256), 0, ctx->stream, ctx->pf.wide, ctx->pf.h_hi, ctx->pf.h_lo,
+                          (size_t)m * ad, 1));
+      if ((s = ug_gemm(ctx, ctx->pf.h_hi, ctx->pf.h_lo, m, ad, dm.adapter_rm, dd, UG_F32, X, nullptr, nullptr, dd))) return s;
       dm.pos_base = m;
     }
     gather_rows_kernel<<<592, 256, 0, ctx->stream>>>(ctx->ids_dev, dm.md.embed, X + (size_t)dm.pos_base * dd, n, dd, V,
@@ -1126,16 +1167,12 @@ spd_status spd_image_adapter(spd_ctx* ctx, const float* feats, int m, int d_in, 
     CU(cudaMemcpyAsync(ia.feats, feats, n_in * sizeof(float), cudaMemcpyHostToDevice, ctx->stream));
     fdev = ia.feats;
   }
-  split_rows_kernel<<<592, 256, 0, ctx->stream>>>(fdev, ia.f_hi, ia.f_lo, n_in);
+  CU(launch_dependent(split_rows_kernel, dim3(592), dim3(256), 0, ctx->stream, fdev, ia.f_hi, ia.f_lo, n_in,
+                      (int)((reinterpret_cast<uintptr_t>(fdev) & 15) == 0)));
   // hidden = GELU(H W1^T), kept as a bf16 hi/lo pair (the GELU runs in the GEMM epilogue)
-  TcArgs a{}; a.M = m; a.N = d_hid; a.K = d_in; a.mode = TC_OUT_SPLIT; a.alpha = 1.f;
-  a.out_hi = ia.g_hi; a.out_lo = ia.g_lo; a.ldo = d_hid;
-  if ((s = tc_gemm(ctx, {ia.f_hi, d_in, m, 1, (size_t)d_in * 2, n_in * 2}, {ia.f_lo, d_in, m, 1, (size_t)d_in * 2, n_in * 2},
-                   {w1, d_in, d_hid, 1, (size_t)d_in * 2, (size_t)d_hid * d_in * 2}, a, true))) return s;
+  if ((s = ug_gemm(ctx, ia.f_hi, ia.f_lo, m, d_in, w1, d_hid, UG_GELU, nullptr, ia.g_hi, ia.g_lo, d_hid))) return s;
   // V = hidden W2^T
-  a = TcArgs{}; a.M = m; a.N = d_out; a.K = d_hid; a.mode = TC_OUT_F32; a.alpha = 1.f; a.out_f32 = out; a.ldo = d_out;
-  if ((s = tc_gemm(ctx, {ia.g_hi, d_hid, m, 1, (size_t)d_hid * 2, n_hid * 2}, {ia.g_lo, d_hid, m, 1, (size_t)d_hid * 2, n_hid * 2},
-                   {w2, d_hid, d_out, 1, (size_t)d_hid * 2, (size_t)d_out * d_hid * 2}, a))) return s;
+  if ((s = ug_gemm(ctx, ia.g_hi, ia.g_lo, m, d_hid, w2, d_out, UG_F32, out, nullptr, nullptr, d_out))) return s;
   // device-side waits are bounded; report one that ran out
   int e = 0;
   CU(cudaMemcpyAsync(&e, &ctx->st->err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
@@ -1417,7 +1454,6 @@ struct spd_batch {
   ModelDev *mds_t = nullptr, *mds_d = nullptr;
   int *rowslot = nullptr, *origins = nullptr, *out_acc = nullptr, *out_next = nullptr;
   float *X = nullptr, *logits = nullptr, *probs = nullptr, *q_all = nullptr, *u_draft = nullptr, *u_verify = nullptr;
-  float* gemm_ws = nullptr;     // partial products of K-sliced GEMMs
   int drafted_gamma = -1;
   int last_rows = 0;
   std::vector<void*> allocs;
@@ -1445,7 +1481,6 @@ spd_status balloc(spd_batch* bt, T** p, size_t n) {
 }
 
 constexpr int BATCH_ATTN_SCRATCH = 100 * 1024;   // two CTAs per SM: 16 warps hide each other's dependency stalls
-constexpr int BATCH_KSPLIT_MAX = 8;
 
 template <int M>
 spd_status launch_batch_attn(spd_ctx* ctx, const ModelDev* mds, const int* origins, int B, int layer, int chain0,
@@ -1456,9 +1491,8 @@ spd_status launch_batch_attn(spd_ctx* ctx, const ModelDev* mds, const int* origi
     CU(cudaFuncSetAttribute((const void*)batch_attn_kernel<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     attr[ctx->device] = true;
   }
-  batch_attn_kernel<M><<<2 * ctx->n_sm, CONSUMER_THREADS, smem, ctx->stream>>>(mds, origins, B, layer, chain0,
-                                                                          BATCH_ATTN_SCRATCH, max_split, o_hi, o_lo);
-  CU(cudaGetLastError());
+  CU(launch_dependent(batch_attn_kernel<M>, dim3(2 * ctx->n_sm), dim3(CONSUMER_THREADS), smem, ctx->stream, mds, origins, B, layer,
+                      chain0, BATCH_ATTN_SCRATCH, max_split, o_hi, o_lo));
   return SPD_OK;
 }
 
@@ -1489,9 +1523,8 @@ spd_status batch_forward(spd_batch* bt, bool draft, int M, int j) {
   cudaStream_t cs = ctx->stream;
   float* X = bt->X;
   const ModelDev* mds = draft ? bt->mds_d : bt->mds_t;
-  batch_embed_kernel<<<R, 128, 0, cs>>>(bt->seqs_dev, B, M, draft ? 1 : 0, j, mh.md.embed, d, V, X, bt->rowslot,
-                                        bt->origins, &ctx->st->err);
-  const Operand h_hi{pf.h_hi, d, R, 1, (size_t)d * 2, (size_t)R * d * 2}, h_lo{pf.h_lo, d, R, 1, (size_t)d * 2, (size_t)R * d * 2};
+  CU(launch_dependent(batch_embed_kernel, dim3(R), dim3(128), 0, cs, bt->seqs_dev, B, M, draft ? 1 : 0, j, mh.md.embed, d, V, X,
+                      bt->rowslot, bt->origins, &ctx->st->err));
   // KV splits per head: about two (sequence, head, split) units per SM, never more than a single
   // sequence would use.  (Choosing the split count for an even division of the units over the CTAs
   // was measured slower: 16 x 32 heads in 2 splits balance better than in 1 but pay for the merges,
@@ -1499,75 +1532,31 @@ spd_status batch_forward(spd_batch* bt, bool draft, int M, int j) {
   int attn_split = (2 * ctx->n_sm + B * H - 1) / (B * H);
   if (attn_split > mh.md.nsplit) attn_split = mh.md.nsplit;
   if (attn_split < 1) attn_split = 1;
-  // every GEMM here is a few rows against a large weight matrix: cut K so that about one CTA per SM streams
-  // K slices: up to one CTA per SM, never a second wave, at least 8 K blocks per slice.  Weight-tile
-  // width (256, 160 or 128 rows): a CTA moves (width + 2 x 128) x K / slices bytes per 64 columns of K
-  // -- its weight rows plus the hi and lo activation tiles -- so the pair (width, slices) that fits
-  // one wave with the fewest bytes per CTA streams fastest; widths whose grid would leave more than
-  // half the SMs without a CTA are not considered.
-  auto slices = [&](int N, int K, int bn) {
-    const int tiles = (N + bn - 1) / bn, kb = (K + TC_BK - 1) / TC_BK;
-    int sp = ctx->n_sm / tiles;
-    if (sp > BATCH_KSPLIT_MAX) sp = BATCH_KSPLIT_MAX;
-    if (sp > kb / 8) sp = kb / 8;
-    return sp < 1 ? 1 : sp;
-  };
-  auto wide = [&](int N, int K) {
-    int best = TC_BN;
-    double best_cost = 0.0;
-    for (int bn : {TC_BN_WIDE, TC_BN_MID, TC_BN}) {
-      const int tiles = (N + bn - 1) / bn, sp = slices(N, K, bn);
-      if (bn != TC_BN && (tiles * sp * 2 < ctx->n_sm || tiles > ctx->n_sm)) continue;
-      const double waves = (double)((tiles * sp + ctx->n_sm - 1) / ctx->n_sm);
-      const double cost = waves * (double)(bn + 2 * TC_BM) * K / sp;
-      if (best_cost == 0.0 || cost < best_cost) { best_cost = cost; best = bn; }
-    }
-    return best;
-  };
-  auto ksplit = [&](int N, int K) { return slices(N, K, wide(N, K)); };
   // Where a projection is cut into K slices, the kernel that reads its result adds the slices up
   // (in slice order): the rotary / cache-append kernel for QKV, the fused residual + RMSNorm + split
   // kernel for the output and down projections.
   const size_t xs = (size_t)R * d;
-  rms_split_kernel<<<R, 256, 0, cs>>>(X, mh.rm[0].attn_norm, mh.cfg.rms_eps, d, pf.h_hi, pf.h_lo);
+  const int rope_blocks = (R * (d >> 3) + 127) / 128;
+  CU(launch_dependent(resid_rms_split_kernel, dim3(R), dim3(256), 0, cs, X, pf.wide, 0, xs, mh.rm[0].attn_norm, mh.cfg.rms_eps, d,
+                      pf.h_hi, pf.h_lo));
   for (int l = 0; l < L; ++l) {
     const ModelHost::RowMajor& w = mh.rm[l];
-    TcArgs a{};
-    a = TcArgs{}; a.M = R; a.N = 3 * d; a.K = d; a.mode = TC_OUT_F32; a.alpha = 1.f; a.out_f32 = pf.wide; a.ldo = 3 * d;
-    const int sq = ksplit(3 * d, d);
-    if ((s = tc_gemm(ctx, h_hi, h_lo, {w.wqkv, d, 3 * d, 1, (size_t)d * 2, (size_t)3 * d * d * 2}, a, false, sq, bt->gemm_ws,
-                     wide(3 * d, d), true))) return s;
-    batch_rope_append_kernel<<<1184, 256, 0, cs>>>(sq > 1 ? bt->gemm_ws : pf.wide, sq, R, M, d, dh, bt->rowslot,
-                                                 mh.md.rope_cos, mh.md.rope_sin, mds, l);
+    int sl = 1;
+    if ((s = ug_gemm(ctx, pf.h_hi, pf.h_lo, R, d, w.wqkv, 3 * d, UG_F32, pf.wide, nullptr, nullptr, 3 * d, UG_SLICES_MAX, &sl))) return s;
+    CU(launch_dependent(batch_rope_append_kernel, dim3(rope_blocks), dim3(128), 0, cs, pf.wide, sl, R, M, d, dh, bt->rowslot,
+                        mh.md.rope_cos, mh.md.rope_sin, mds, l));
     // (the attention kernel leaves its rows as the hi/lo operand of the output projection)
     if ((s = batch_attn(ctx, M, mds, bt->origins, B, l, draft ? j - 1 : 0, attn_split, pf.h_hi, pf.h_lo))) return s;
-    a = TcArgs{}; a.M = R; a.N = d; a.K = d; a.mode = TC_OUT_F32_ADD; a.alpha = 1.f; a.out_f32 = X; a.ldo = d;
-    const int so = ksplit(d, d);
-    if ((s = tc_gemm(ctx, h_hi, h_lo, {w.wo, d, d, 1, (size_t)d * 2, (size_t)d * d * 2}, a, false, so, bt->gemm_ws, wide(d, d),
-                     true))) return s;
-    resid_rms_split_kernel<<<R, 256, 0, cs>>>(X, bt->gemm_ws, so > 1 ? so : 0, xs, w.ffn_norm, mh.cfg.rms_eps, d, pf.h_hi, pf.h_lo);
-    const int sg = ksplit(2 * f, d);
-    if (sg == 1) {   // SwiGLU in the GEMM's epilogue
-      a = TcArgs{}; a.M = R; a.N = 2 * f; a.K = d; a.mode = TC_OUT_SWIGLU; a.alpha = 1.f; a.out_hi = pf.g_hi; a.out_lo = pf.g_lo; a.ldo = f;
-      if ((s = tc_gemm(ctx, h_hi, h_lo, {w.wgu, d, 2 * f, 1, (size_t)d * 2, (size_t)2 * f * d * 2}, a, false, 1, bt->gemm_ws,
-                       wide(2 * f, d)))) return s;
-    } else {
-      a = TcArgs{}; a.M = R; a.N = 2 * f; a.K = d; a.mode = TC_OUT_F32; a.alpha = 1.f; a.out_f32 = pf.wide; a.ldo = 2 * f;
-      if ((s = tc_gemm(ctx, h_hi, h_lo, {w.wgu, d, 2 * f, 1, (size_t)d * 2, (size_t)2 * f * d * 2}, a, false, sg, bt->gemm_ws,
-                       wide(2 * f, d)))) return s;
-      swiglu_split_kernel<<<296, 256, 0, cs>>>(pf.wide, R, f, pf.g_hi, pf.g_lo);
-    }
-    a = TcArgs{}; a.M = R; a.N = d; a.K = f; a.mode = TC_OUT_F32_ADD; a.alpha = 1.f; a.out_f32 = X; a.ldo = d;
-    const int sd = ksplit(d, f);
-    if ((s = tc_gemm(ctx, {pf.g_hi, f, R, 1, (size_t)f * 2, (size_t)R * f * 2}, {pf.g_lo, f, R, 1, (size_t)f * 2, (size_t)R * f * 2},
-                     {w.wd, f, d, 1, (size_t)f * 2, (size_t)d * f * 2}, a, false, sd, bt->gemm_ws, wide(d, f), true))) return s;
+    if ((s = ug_gemm(ctx, pf.h_hi, pf.h_lo, R, d, w.wo, d, UG_F32, pf.wide, nullptr, nullptr, d, UG_SLICES_MAX, &sl))) return s;
+    CU(launch_dependent(resid_rms_split_kernel, dim3(R), dim3(256), 0, cs, X, pf.wide, sl, xs, w.ffn_norm, mh.cfg.rms_eps, d, pf.h_hi,
+                        pf.h_lo));
+    if ((s = ug_gemm(ctx, pf.h_hi, pf.h_lo, R, d, w.wgu, 2 * f, UG_SWIGLU, nullptr, pf.g_hi, pf.g_lo, f))) return s;
+    if ((s = ug_gemm(ctx, pf.g_hi, pf.g_lo, R, f, w.wd, d, UG_F32, pf.wide, nullptr, nullptr, d, UG_SLICES_MAX, &sl))) return s;
     // the norm in front of the next layer (or of the LM head) rides on the residual update
-    resid_rms_split_kernel<<<R, 256, 0, cs>>>(X, bt->gemm_ws, sd > 1 ? sd : 0, xs,
-                                              l + 1 < L ? mh.rm[l + 1].attn_norm : mh.md.final_norm, mh.cfg.rms_eps, d,
-                                              pf.h_hi, pf.h_lo);
+    CU(launch_dependent(resid_rms_split_kernel, dim3(R), dim3(256), 0, cs, X, pf.wide, sl, xs,
+                        l + 1 < L ? mh.rm[l + 1].attn_norm : mh.md.final_norm, mh.cfg.rms_eps, d, pf.h_hi, pf.h_lo));
   }
-  TcArgs a{}; a.M = R; a.N = V; a.K = d; a.mode = TC_OUT_F32; a.alpha = 1.f; a.out_f32 = bt->logits; a.ldo = V;
-  if ((s = tc_gemm(ctx, h_hi, h_lo, {mh.lm_rm, d, V, 1, (size_t)d * 2, (size_t)V * d * 2}, a, false, ksplit(V, d), bt->gemm_ws, wide(V, d)))) return s;
+  if ((s = ug_gemm(ctx, pf.h_hi, pf.h_lo, R, d, mh.lm_rm, V, UG_F32, bt->logits, nullptr, nullptr, V))) return s;
   CU(cudaGetLastError());
   bt->last_rows = R;
   return SPD_OK;
@@ -1577,7 +1566,7 @@ spd_status batch_forward(spd_batch* bt, bool draft, int M, int j) {
 spd_status batch_probs(spd_batch* bt, int R) {
   spd_ctx* ctx = bt->lead;
   const int V = ctx->cfg.target.vocab;
-  batch_softmax_kernel<<<R, SAMPLE_THREADS, 0, ctx->stream>>>(bt->logits, V, ctx->cfg.temperature, bt->probs);
+  CU(launch_dependent(batch_softmax_kernel, dim3(R), dim3(SAMPLE_THREADS), 0, ctx->stream, bt->logits, V, ctx->cfg.temperature, bt->probs));
   if (ctx->truncate)
     truncate_rows_kernel<<<R, WARP_THREADS, (size_t)V * sizeof(float), ctx->stream>>>(
         bt->probs, bt->probs, V, ctx->cfg.top_k, ctx->cfg.top_p > 0.f ? ctx->cfg.top_p : 1.0f);
@@ -1687,14 +1676,6 @@ spd_status spd_batch_create(spd_ctx* const* seqs, int B, spd_batch** out) {
   if (!s) s = balloc(bt, &bt->q_all, (size_t)B * gm * V);
   if (!s) s = balloc(bt, &bt->u_draft, (size_t)B * MAX_M);
   if (!s) s = balloc(bt, &bt->u_verify, (size_t)B * MAX_M);
-  {   // widest split output: [slices][128 rows][max(3 d, 2 f, V)]
-    size_t wide = (size_t)V;
-    for (const spd_model_cfg* c : {&ctx->cfg.target, &ctx->cfg.draft}) {
-      if ((size_t)3 * c->d_model > wide) wide = (size_t)3 * c->d_model;
-      if ((size_t)2 * c->d_ffn > wide) wide = (size_t)2 * c->d_ffn;
-    }
-    if (!s) s = balloc(bt, &bt->gemm_ws, (size_t)BATCH_KSPLIT_MAX * BATCH_ROWS_MAX * wide);
-  }
   if (!s && ctx->truncate &&
       cudaFuncSetAttribute((const void*)truncate_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)((size_t)V * sizeof(float))) != cudaSuccess)
@@ -1738,9 +1719,8 @@ spd_status spd_batch_draft(spd_batch* bt, int gamma, const float* uniforms, int3
       spd_status r;
       if ((r = batch_forward(bt, true, 2, j))) return r;
       if (!ctx->cfg.greedy && (r = batch_probs(bt, 2 * B))) return r;
-      batch_draft_sample_kernel<<<B, SAMPLE_THREADS, 0, ctx->stream>>>(
-          bt->seqs_dev, ctx->cfg.greedy ? bt->logits : bt->probs, V, gamma, j, ctx->cfg.greedy, bt->u_draft, bt->q_all);
-      CU(cudaGetLastError());
+      CU(launch_dependent(batch_draft_sample_kernel, dim3(B), dim3(SAMPLE_THREADS), 0, ctx->stream, bt->seqs_dev,
+                          ctx->cfg.greedy ? bt->logits : bt->probs, V, gamma, j, ctx->cfg.greedy, bt->u_draft, bt->q_all));
       return SPD_OK;
     };
     if ((s = run_step_graph(bt, bt->g_draft[gamma][j], step))) return s;
@@ -1772,10 +1752,9 @@ spd_status spd_batch_verify(spd_batch* bt, int gamma, const float* uniforms, int
     spd_status r;
     if ((r = batch_forward(bt, false, M, 0))) return r;
     if (!ctx->cfg.greedy && (r = batch_probs(bt, B * M))) return r;
-    batch_verify_kernel<<<B, SAMPLE_THREADS, 0, ctx->stream>>>(bt->seqs_dev, ctx->cfg.greedy ? bt->logits : bt->probs,
-                                                                bt->q_all, ctx->cfg.greedy ? nullptr : bt->u_verify, gamma,
-                                                                V, ctx->cfg.greedy, bt->out_acc, bt->out_next);
-    CU(cudaGetLastError());
+    CU(launch_dependent(batch_verify_kernel, dim3(B), dim3(SAMPLE_THREADS), 0, ctx->stream, bt->seqs_dev,
+                        ctx->cfg.greedy ? bt->logits : bt->probs, bt->q_all, ctx->cfg.greedy ? nullptr : bt->u_verify, gamma, V,
+                        ctx->cfg.greedy, bt->out_acc, bt->out_next));
     return SPD_OK;
   };
   if ((s = run_step_graph(bt, bt->g_verify[gamma], step))) return s;

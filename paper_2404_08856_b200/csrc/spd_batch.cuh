@@ -7,6 +7,7 @@
 // its own length and its own accepted count (Sec. 2.1's rule is stated per sequence).
 #pragma once
 #include "spd_kernel.cuh"
+#include "spd_prefill.cuh"
 
 namespace spd {
 
@@ -23,6 +24,8 @@ constexpr int BATCH_ROWS_MAX = 128;   // one 128-row tile of the tensor-core GEM
 // absolute cache row, and each sequence's origin.  An id outside [0, V) is read as 0 and reported.
 __global__ void batch_embed_kernel(const BatchSeq* seqs, int B, int M, int draft, int j, const float* table, int d,
                                    int V, float* X, int* rowslot, int* origins, int* err) {
+  pdl_wait();
+  pdl_trigger();
   const int r = blockIdx.x, b = r / M, m = r - b * M;
   const DevState* st = seqs[b].st;
   const int origin = (draft ? seqs[b].pos_base_d : seqs[b].pos_base_t) + st->n_text;
@@ -45,41 +48,31 @@ __global__ void batch_embed_kernel(const BatchSeq* seqs, int B, int M, int draft
   for (int i = threadIdx.x; i < (d >> 2); i += blockDim.x) dst[i] = src[i];
 }
 
-// qkv fp32 [R][3d] (natural row order) -> rotary embedding on q and k at each row's own position
-// (pairs (i, i + dh/2)); q goes to its sequence's query rows [M][d] (fp32), k and v are appended
-// to its sequence's cache at the row's cache row.
-// `qkv` may be the sum of `slices` partial products [slices][R][3d] (K slices of the projection, added in
-// slice order as tc_reduce_kernel does).
+// qkv [slices][R][3d] (natural row order; K slices of the projection, added in slice order) -> rotary
+// embedding on q and k at each row's own position; q goes to its sequence's query rows [M][d]
+// (fp32), k and v are appended to its sequence's cache at the row's cache row.
 __global__ void batch_rope_append_kernel(const float* qkv, int slices, int R, int M, int d, int dh, const int* rowslot,
                                          const float* cs, const float* sn, const ModelDev* mds, int layer) {
-  const size_t sstride = (size_t)R * 3 * d;
-  auto at = [&](const float* p) {
-    float v = 0.f;
-    for (int s = 0; s < slices; ++s) v += p[(size_t)s * sstride];
-    return v;
-  };
-  const int half = dh >> 1, pairs = d >> 1;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < (size_t)R * pairs;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const int r = (int)(i / pairs), p = (int)(i - (size_t)r * pairs);
-    const int b = r / M, m = r - b * M;
-    const int h = p / half, jj = p - h * half;
-    const int c0 = h * dh + jj, c1 = c0 + half;
-    const int pos = rowslot[r];
-    const float* row = qkv + (size_t)r * 3 * d;
-    const float c = cs[(size_t)pos * half + jj], s = sn[(size_t)pos * half + jj];
-    const float qa = at(row + c0), qb = at(row + c1), ka = at(row + d + c0), kb = at(row + d + c1);
+  pdl_wait();
+  pdl_trigger();
+  const int half = dh >> 1, quads = d >> 3, per_head = half >> 2;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < R * quads; i += gridDim.x * blockDim.x) {
+    const int r = i / quads, g = i - r * quads, h = g / per_head, j = (g - h * per_head) << 2, c0 = h * dh + j;
+    const int b = r / M, m = r - b * M, pos = rowslot[r];
     const ModelDev& md = mds[b];
-    float* q = md.qbuf + (size_t)m * d;
-    q[c0] = qa * c - qb * s;
-    q[c1] = qb * c + qa * s;
-    const size_t crow = (((size_t)layer * md.H + h) * md.max_seq + pos) * dh;   // cache: [L][H][max_seq][dh]
+    const float4 c = *reinterpret_cast<const float4*>(cs + (size_t)pos * half + j);
+    const float4 s = *reinterpret_cast<const float4*>(sn + (size_t)pos * half + j);
+    const RopeQuad o = rope_quad(qkv, slices, (size_t)R * 3 * d, r, d, c0, half, c, s);
+    float* q = md.qbuf + (size_t)m * d + c0;
+    *reinterpret_cast<float4*>(q) = o.qa;
+    *reinterpret_cast<float4*>(q + half) = o.qb;
+    const size_t crow = (((size_t)layer * md.H + h) * md.max_seq + pos) * dh + j;   // cache: [L][H][max_seq][dh]
     __nv_bfloat16* kc = static_cast<__nv_bfloat16*>(md.kcache) + crow;
     __nv_bfloat16* vc = static_cast<__nv_bfloat16*>(md.vcache) + crow;
-    kc[jj] = __float2bfloat16_rn(ka * c - kb * s);
-    kc[jj + half] = __float2bfloat16_rn(kb * c + ka * s);
-    vc[jj] = __float2bfloat16_rn(at(row + 2 * d + c0));
-    vc[jj + half] = __float2bfloat16_rn(at(row + 2 * d + c1));
+    *reinterpret_cast<uint2*>(kc) = pack4(o.ka);
+    *reinterpret_cast<uint2*>(kc + half) = pack4(o.kb);
+    *reinterpret_cast<uint2*>(vc) = pack4(o.va);
+    *reinterpret_cast<uint2*>(vc + half) = pack4(o.vb);
   }
 }
 
@@ -98,6 +91,8 @@ __global__ void __launch_bounds__(CONSUMER_THREADS, 2) batch_attn_kernel(const M
                                                                       int layer, int chain0, int xbytes, int max_split,
                                                                       __nv_bfloat16* o_hi, __nv_bfloat16* o_lo) {
   extern __shared__ __align__(1024) char bsm[];
+  pdl_wait();
+  pdl_trigger();
   Ctrl* ctl = reinterpret_cast<Ctrl*>(bsm);
   char* xs = bsm + CTRL_BYTES;
   if (threadIdx.x < M) {
@@ -124,6 +119,8 @@ __global__ void __launch_bounds__(CONSUMER_THREADS, 2) batch_attn_kernel(const M
 __global__ void __launch_bounds__(SAMPLE_THREADS) batch_softmax_kernel(const float* logits, int V, float temperature,
                                                                        float* probs) {
   __shared__ float red[8];
+  pdl_wait();
+  pdl_trigger();
   const float* row = logits + (size_t)blockIdx.x * V;
   float* out = probs + (size_t)blockIdx.x * V;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -157,6 +154,8 @@ __global__ void __launch_bounds__(SAMPLE_THREADS) batch_draft_sample_kernel(cons
                                                                             int V, int gamma, int j, int greedy,
                                                                             const float* u, float* q_all) {
   __shared__ SampleScratch sc;
+  pdl_wait();
+  pdl_trigger();
   const int b = blockIdx.x;
   const float* row = rows + ((size_t)b * 2 + 1) * V;
   int tok;
@@ -178,6 +177,8 @@ __global__ void __launch_bounds__(SAMPLE_THREADS) batch_verify_kernel(const Batc
                                                                       int V, int greedy, int* n_acc, int* next) {
   __shared__ SampleScratch sc;
   __shared__ int s_ids[MAX_M];
+  pdl_wait();
+  pdl_trigger();
   const int b = blockIdx.x;
   DevState* st = seqs[b].st;
   if (threadIdx.x < gamma) {

@@ -98,6 +98,14 @@ __device__ __forceinline__ uint64_t policy_evict_first() {
   return p;
 }
 
+// Dependent launch (programmatic stream serialisation): a kernel launched that way may start while
+// its predecessor still runs; pdl_wait returns once the predecessor has finished and its writes are
+// visible.  Every such kernel calls pdl_wait in every CTA before it touches anything an earlier
+// kernel writes, so waiting for the predecessor covers all kernels before it.  pdl_trigger lets the
+// successor start (as its CTAs find room).  Both do nothing in an ordinary launch.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Named barrier among the first `n` threads' warps (id 1..15; 0 is __syncthreads).
 __device__ __forceinline__ void named_sync(int id, int n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
