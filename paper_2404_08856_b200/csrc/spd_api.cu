@@ -251,7 +251,6 @@ spd_status alloc_sequence_state(spd_ctx* ctx, ModelHost& mh) {
   if ((s = dalloc(ctx, &md.aml, (size_t)H * md.nsplit * MAX_M * 2))) return s;
   if ((s = dalloc(ctx, &md.head_cnt, (size_t)H))) return s;
   if ((s = dalloc(ctx, &md.stat_part, (size_t)ctx->n_sm * MAX_M * 4))) return s;
-  if ((s = dalloc(ctx, &md.cdf_part, (size_t)ctx->n_sm * 2 + 2))) return s;
   if ((s = dalloc(ctx, &mh.logits, (size_t)MAX_M * V))) return s;
   return SPD_OK;
 }
@@ -464,6 +463,35 @@ bool cluster_fits(KernelFn fn, int cs, size_t smem) {
   return n >= 1;
 }
 
+// A launch of `rows` clusters of C CTAs (the sampling kernels).
+template <class... KA, class... A>
+cudaError_t launch_rows(void (*kernel)(KA...), int rows, int C, int threads, cudaStream_t stream, bool dependent, A&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(rows * C); cfg.blockDim = dim3(threads); cfg.stream = stream;
+  cudaLaunchAttribute at[2];
+  int n = 0;
+  if (C > 1) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = C; at[n].val.clusterDim.y = 1; at[n].val.clusterDim.z = 1;
+    ++n;
+  }
+  if (dependent) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+  }
+  cfg.attrs = at; cfg.numAttrs = n;
+  return cudaLaunchKernelEx(&cfg, kernel, KA(args)...);
+}
+
+// CTAs per row: as many as keep all rows on the device at once, at most 8 (the portable cluster size), and
+// none with less than ~1000 entries of the row (a CTA's fixed cost is then larger than its share).
+int row_ctas(int n_sm, int rows, int V) {
+  int C = ROW_CTAS_MAX;
+  while (C > 1 && (rows * C > n_sm || V / C < ROW_THREADS)) C >>= 1;
+  return C;
+}
+
 // grid = CTAs of the launch; cluster > 0: they form one thread-block cluster (then grid == cluster)
 // and synchronise inside it, otherwise it is a cooperative launch with the barrier word `bar`.
 spd_status launch_forward(spd_ctx* ctx, int M, int dtype, StepArgs a, cudaStream_t stream, int grid, int cluster,
@@ -490,20 +518,20 @@ spd_status launch_forward(spd_ctx* ctx, int M, int dtype, StepArgs a, cudaStream
     CU(cudaMemsetAsync(bar, 0, sizeof(unsigned), stream));
     CU(cudaLaunchCooperativeKernel((const void*)fn, dim3(grid), dim3(ENGINE_THREADS), params, lc.smem, stream));
   }
-  // sampling (not greedy): the forward kernel has left logits and per-slice row statistics; two
-  // small kernels spread the draw over the whole device and commit the step
+  // sampling (not greedy): the forward kernel has left logits and per-slice row statistics; a small
+  // kernel on one cluster makes the draw and commits the step
   const bool samples = a.mode == MODE_VERIFY || a.mode == MODE_DRAFT || (a.mode == MODE_ROWS && a.want_sample);
   if (samples && !a.greedy && !a.tree) {
+    const int C = row_ctas(n_sm_sampling, 1, a.md.V);
     if (ctx && ctx->truncate) {
       // top-k / top-p: probability rows -> truncated and renormalised in place -> the rule on rows
       const int nrows = a.mode == MODE_VERIFY ? a.gamma + 1 : 1;
-      prob_rows_kernel<<<n_sm_sampling, SAMPLE_THREADS, 0, stream>>>(a, ctx->prow);
+      prob_rows_kernel<<<n_sm_sampling, PROB_THREADS, 0, stream>>>(a, ctx->prow);
       truncate_rows_kernel<<<nrows, WARP_THREADS, (size_t)a.md.V * sizeof(float), stream>>>(
           ctx->prow, ctx->prow, a.md.V, ctx->cfg.top_k, ctx->cfg.top_p > 0.f ? ctx->cfg.top_p : 1.0f);
-      sample_rows_kernel<<<1, SAMPLE_THREADS, 0, stream>>>(a, ctx->prow);
+      CU(launch_rows(sample_rows_kernel, 1, C, ROW_THREADS, stream, false, a, C, ctx->prow));
     } else {
-      sample_slices_kernel<<<n_sm_sampling, SAMPLE_THREADS, 0, stream>>>(a);
-      sample_pick_kernel<<<1, SAMPLE_THREADS, 0, stream>>>(a, n_sm_sampling);
+      CU(launch_rows(sample_step_kernel, 1, C, ROW_THREADS, stream, false, a, C));
     }
     CU(cudaGetLastError());
   }
@@ -1297,7 +1325,7 @@ static spd_status tree_shape_from_parent(spd_ctx* ctx, int n, const int32_t* par
 
 // probability rows of the launch's statistic rows (truncated when top-k / top-p is on)
 static spd_status tree_prob_rows(spd_ctx* ctx, const StepArgs& a, cudaStream_t stream) {
-  prob_rows_kernel<<<ctx->n_sm, SAMPLE_THREADS, 0, stream>>>(a, ctx->prow);
+  prob_rows_kernel<<<ctx->n_sm, PROB_THREADS, 0, stream>>>(a, ctx->prow);
   if (ctx->truncate)
     truncate_rows_kernel<<<a.stat_n, WARP_THREADS, (size_t)a.md.V * sizeof(float), stream>>>(
         ctx->prow, ctx->prow, a.md.V, ctx->cfg.top_k, ctx->cfg.top_p > 0.f ? ctx->cfg.top_p : 1.0f);
@@ -1359,9 +1387,9 @@ spd_status spd_draft_tree(spd_ctx* ctx, int depth, const int32_t* branching, con
     }
     if ((s = launch_model(ctx, dm, M, a, ctx->stream))) return s;
     a.fwd_grid = dm.grid; a.sample_r0 = M - 1;
-    if (!ctx->cfg.greedy && (s = tree_prob_rows(ctx, a, ctx->stream))) return s;
-    tree_draw_kernel<<<1, SAMPLE_THREADS, 0, ctx->stream>>>(a, sh, ctx->prow);
-    CU(cudaGetLastError());
+    if (ctx->truncate && (s = tree_prob_rows(ctx, a, ctx->stream))) return s;
+    const int C = row_ctas(ctx->n_sm, a.stat_n, dm.cfg.vocab);
+    CU(launch_rows(tree_draw_kernel, a.stat_n, C, ROW_THREADS, ctx->stream, false, a, sh, C, ctx->prow, (int)ctx->truncate));
   }
   ctx->tree_shape = sh;
   ctx->tree_drafted = true;
@@ -1419,7 +1447,7 @@ spd_status spd_verify_tree(spd_ctx* ctx, int n_nodes, const int32_t* parent, con
   if ((s = launch_model(ctx, tm, n + 1, a, ctx->stream))) return s;
   a.fwd_grid = tm.grid; a.sample_r0 = n;
   if (!ctx->cfg.greedy && (s = tree_prob_rows(ctx, a, ctx->stream))) return s;
-  tree_verify_kernel<<<1, SAMPLE_THREADS, 0, ctx->stream>>>(a, sh, ctx->prow, ctx->tree_cur);
+  tree_verify_kernel<<<1, ROW_THREADS, 0, ctx->stream>>>(a, sh, ctx->prow, ctx->tree_cur);
   // accepted rows move up to the positions they now hold, in both caches (the draft was fed the
   // nodes above the deepest level only)
   for (int pass = 0; pass < 2; ++pass) {
@@ -1453,6 +1481,7 @@ struct spd_batch {
   BatchSeq* seqs_dev = nullptr;
   ModelDev *mds_t = nullptr, *mds_d = nullptr;
   int *rowslot = nullptr, *origins = nullptr, *out_acc = nullptr, *out_next = nullptr;
+  RowStats* stats = nullptr;    // (max, sum exp) of the rows of a verify step
   float *X = nullptr, *logits = nullptr, *probs = nullptr, *q_all = nullptr, *u_draft = nullptr, *u_verify = nullptr;
   int drafted_gamma = -1;
   int last_rows = 0;
@@ -1562,13 +1591,15 @@ spd_status batch_forward(spd_batch* bt, bool draft, int M, int j) {
   return SPD_OK;
 }
 
-// softmax rows of bt->logits -> bt->probs, truncated when top-k / top-p is on
-spd_status batch_probs(spd_batch* bt, int R) {
+// statistics of rows first, first + stride, ... of bt->logits; with top-k / top-p on also their truncated
+// probability rows in bt->probs
+spd_status batch_probs(spd_batch* bt, int rows, int first, int stride) {
   spd_ctx* ctx = bt->lead;
   const int V = ctx->cfg.target.vocab;
-  CU(launch_dependent(batch_softmax_kernel, dim3(R), dim3(SAMPLE_THREADS), 0, ctx->stream, bt->logits, V, ctx->cfg.temperature, bt->probs));
+  CU(launch_rows(batch_softmax_kernel, rows, 1, ROW_THREADS, ctx->stream, true, bt->logits, first, stride, V, ctx->cfg.temperature, bt->stats,
+                 ctx->truncate ? bt->probs : nullptr));
   if (ctx->truncate)
-    truncate_rows_kernel<<<R, WARP_THREADS, (size_t)V * sizeof(float), ctx->stream>>>(
+    truncate_rows_kernel<<<rows, WARP_THREADS, (size_t)V * sizeof(float), ctx->stream>>>(
         bt->probs, bt->probs, V, ctx->cfg.top_k, ctx->cfg.top_p > 0.f ? ctx->cfg.top_p : 1.0f);
   CU(cudaGetLastError());
   return SPD_OK;
@@ -1672,7 +1703,8 @@ spd_status spd_batch_create(spd_ctx* const* seqs, int B, spd_batch** out) {
   if (!s) s = balloc(bt, &bt->out_next, (size_t)B);
   if (!s) s = balloc(bt, &bt->X, (size_t)BATCH_ROWS_MAX * dmax);
   if (!s) s = balloc(bt, &bt->logits, (size_t)BATCH_ROWS_MAX * V);
-  if (!s) s = balloc(bt, &bt->probs, (size_t)BATCH_ROWS_MAX * V);
+  if (!s) s = balloc(bt, &bt->stats, (size_t)BATCH_ROWS_MAX);
+  if (!s && ctx->truncate) s = balloc(bt, &bt->probs, (size_t)BATCH_ROWS_MAX * V);
   if (!s) s = balloc(bt, &bt->q_all, (size_t)B * gm * V);
   if (!s) s = balloc(bt, &bt->u_draft, (size_t)B * MAX_M);
   if (!s) s = balloc(bt, &bt->u_verify, (size_t)B * MAX_M);
@@ -1718,9 +1750,10 @@ spd_status spd_batch_draft(spd_batch* bt, int gamma, const float* uniforms, int3
     auto step = [&]() -> spd_status {
       spd_status r;
       if ((r = batch_forward(bt, true, 2, j))) return r;
-      if (!ctx->cfg.greedy && (r = batch_probs(bt, 2 * B))) return r;
-      CU(launch_dependent(batch_draft_sample_kernel, dim3(B), dim3(SAMPLE_THREADS), 0, ctx->stream, bt->seqs_dev,
-                          ctx->cfg.greedy ? bt->logits : bt->probs, V, gamma, j, ctx->cfg.greedy, bt->u_draft, bt->q_all));
+      // (each sequence's first row only refreshes the cache: nothing is drawn from it)
+      if (ctx->truncate && (r = batch_probs(bt, B, 1, 2))) return r;
+      CU(launch_rows(batch_draft_sample_kernel, B, 1, ROW_THREADS, ctx->stream, true, bt->seqs_dev, bt->logits,
+                     ctx->truncate ? bt->probs : nullptr, V, gamma, j, ctx->cfg.greedy, ctx->cfg.temperature, bt->u_draft, bt->q_all));
       return SPD_OK;
     };
     if ((s = run_step_graph(bt, bt->g_draft[gamma][j], step))) return s;
@@ -1751,10 +1784,11 @@ spd_status spd_batch_verify(spd_batch* bt, int gamma, const float* uniforms, int
   auto step = [&]() -> spd_status {
     spd_status r;
     if ((r = batch_forward(bt, false, M, 0))) return r;
-    if (!ctx->cfg.greedy && (r = batch_probs(bt, B * M))) return r;
-    CU(launch_dependent(batch_verify_kernel, dim3(B), dim3(SAMPLE_THREADS), 0, ctx->stream, bt->seqs_dev,
-                        ctx->cfg.greedy ? bt->logits : bt->probs, bt->q_all, ctx->cfg.greedy ? nullptr : bt->u_verify, gamma, V,
-                        ctx->cfg.greedy, bt->out_acc, bt->out_next));
+    if (!ctx->cfg.greedy && (r = batch_probs(bt, B * M, 0, 1))) return r;
+    const int C = row_ctas(ctx->n_sm, B, V);
+    CU(launch_rows(batch_verify_kernel, B, C, ROW_THREADS, ctx->stream, true, bt->seqs_dev, C, bt->logits, bt->stats,
+                   ctx->truncate ? bt->probs : nullptr, bt->q_all, ctx->cfg.greedy ? nullptr : bt->u_verify, gamma, V,
+                   ctx->cfg.greedy, ctx->cfg.temperature, bt->out_acc, bt->out_next));
     return SPD_OK;
   };
   if ((s = run_step_graph(bt, bt->g_verify[gamma], step))) return s;
@@ -1962,9 +1996,15 @@ spd_status spd_reject_sample(const float* p, const float* q, const int32_t* ids,
   if (!p || !n_acc || !next || B < 1 || gamma < 0 || V < 1) return SPD_EINVAL;
   if (gamma > 0 && !ids) return SPD_EINVAL;
   if (!greedy && (!u || (gamma > 0 && !q))) return SPD_EINVAL;
-  reject_sample_kernel<<<B, SAMPLE_THREADS, 0, static_cast<cudaStream_t>(stream)>>>(p, q, ids, u, gamma, V, greedy,
-                                                                                    n_acc, next);
-  return cudaGetLastError() == cudaSuccess ? SPD_OK : SPD_ECUDA;
+  int dev = 0, n_sm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return SPD_ECUDA;
+  // four entries of the row per thread: with a small vocabulary many sequences share an SM
+  const int C = row_ctas(n_sm, B, V);
+  int threads = ((V / C + 3) / 4 + 31) / 32 * 32;
+  if (threads > ROW_THREADS) threads = ROW_THREADS;
+  return launch_rows(reject_sample_kernel, B, C, threads, static_cast<cudaStream_t>(stream), false, p, q, ids, u, gamma, V, greedy, C, n_acc,
+                     next) == cudaSuccess ? SPD_OK : SPD_ECUDA;
 }
 
 spd_status spd_truncate_probs(const float* probs, float* out, int rows, int V, int top_k, float top_p, void* stream) {

@@ -114,82 +114,111 @@ __global__ void __launch_bounds__(CONSUMER_THREADS, 2) batch_attn_kernel(const M
   }
 }
 
-// softmax(logits / T) of each row (one CTA per row), the same arithmetic per element as the
-// single-sequence path: exp(l / T - max) / sum, each step one IEEE operation.
-__global__ void __launch_bounds__(SAMPLE_THREADS) batch_softmax_kernel(const float* logits, int V, float temperature,
-                                                                       float* probs) {
-  __shared__ float red[8];
-  pdl_wait();
-  pdl_trigger();
-  const float* row = logits + (size_t)blockIdx.x * V;
-  float* out = probs + (size_t)blockIdx.x * V;
+// ---- sampling.  CTAs of ROW_THREADS threads per row or sequence (a batch has enough of them to fill
+// the device); the row is read from L2 a few times instead of being kept anywhere.
+
+// max and sum of exp of logits / T over a row, each step one IEEE operation (as the single-sequence path)
+struct RowStats { float mx, sum; };
+__device__ RowStats row_stats(const float* row, int V, float T, float* red /*[ROW_WARPS]*/) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float mx = -INFINITY;
-  for (int k = threadIdx.x; k < V; k += SAMPLE_THREADS) mx = fmaxf(mx, __fdiv_rn(row[k], temperature));
+#pragma unroll 8
+  for (int k = threadIdx.x; k < V; k += ROW_THREADS) mx = fmaxf(mx, __fdiv_rn(ldcg(row + k), T));
 #pragma unroll
   for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   if (lane == 0) red[warp] = mx;
   __syncthreads();
-  mx = red[0];
+  mx = red[lane];
 #pragma unroll
-  for (int w = 1; w < 8; ++w) mx = fmaxf(mx, red[w]);
+  for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   __syncthreads();
   float sum = 0.f;
-  for (int k = threadIdx.x; k < V; k += SAMPLE_THREADS) sum += expf(__fsub_rn(__fdiv_rn(row[k], temperature), mx));
+#pragma unroll 8
+  for (int k = threadIdx.x; k < V; k += ROW_THREADS) sum += expf(__fsub_rn(__fdiv_rn(ldcg(row + k), T), mx));
 #pragma unroll
   for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
   if (lane == 0) red[warp] = sum;
   __syncthreads();
-  float tot = 0.f;
+  sum = red[lane];
 #pragma unroll
-  for (int w = 0; w < 8; ++w) tot += red[w];
-  for (int k = threadIdx.x; k < V; k += SAMPLE_THREADS)
-    out[k] = __fdiv_rn(expf(__fsub_rn(__fdiv_rn(row[k], temperature), mx)), tot);
+  for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  return RowStats{mx, sum};
 }
 
-// Draft step j of every sequence (one CTA each): x_j drawn from the sequence's row of q_j (rows
-// [B][2][V], the second row of a sequence is the token being extended), or its arg-max of the
-// logits when greedy; q_j is kept as row j of the sequence's draft distributions [B][gamma][V].
-__global__ void __launch_bounds__(SAMPLE_THREADS) batch_draft_sample_kernel(const BatchSeq* seqs, const float* rows,
-                                                                            int V, int gamma, int j, int greedy,
-                                                                            const float* u, float* q_all) {
-  __shared__ SampleScratch sc;
+// (max, sum exp) of every row -> stats [rows]; with probs also the probability rows (the truncated path
+// needs them whole).  Row i reads logits row first + i * stride.
+__global__ void __launch_bounds__(ROW_THREADS) batch_softmax_kernel(const float* logits, int first, int stride, int V,
+                                                                    float temperature, RowStats* stats, float* probs) {
+  __shared__ float red[ROW_WARPS];
+  pdl_wait();
+  pdl_trigger();
+  const float* row = logits + ((size_t)first + (size_t)blockIdx.x * stride) * V;
+  const RowStats rs = row_stats(row, V, temperature, red);
+  if (threadIdx.x == 0) stats[blockIdx.x] = rs;
+  if (probs) {
+    float* out = probs + (size_t)blockIdx.x * V;
+#pragma unroll 8
+    for (int k = threadIdx.x; k < V; k += ROW_THREADS) out[k] = prob_of(ldcg(row + k), temperature, rs.mx, rs.sum);
+  }
+}
+
+// Draft step j of every sequence (one CTA each): x_j drawn from q_j = softmax(logits / T) of the sequence's
+// second row (the token being extended), or its arg-max when greedy; q_j is kept as row j of the
+// sequence's draft distributions [B][gamma][V].  probs: the truncated rows [B][V], or NULL.
+__global__ void __launch_bounds__(ROW_THREADS) batch_draft_sample_kernel(const BatchSeq* seqs, const float* logits,
+                                                                         const float* probs, int V, int gamma, int j, int greedy,
+                                                                         float temperature, const float* u, float* q_all) {
+  __shared__ RowScratch sc;
+  __shared__ float red[ROW_WARPS];
   pdl_wait();
   pdl_trigger();
   const int b = blockIdx.x;
-  const float* row = rows + ((size_t)b * 2 + 1) * V;
+  const RowSlice rs{0, 1};
+  const float* lrow = logits + ((size_t)b * 2 + 1) * V;
   int tok;
   if (greedy) {
-    tok = block_argmax([&](int k) { return row[k]; }, V, &sc);
+    rows_argmax([&](int, int k) { return ldcg(lrow + k); }, 1, V, rs, &sc);
+    tok = sc.arg[0];
   } else {
-    tok = block_sample([&](int k) { return row[k]; }, V, u[(size_t)b * gamma + j], &sc);
+    const float* prow = probs ? probs + (size_t)b * V : nullptr;
+    const RowStats st = probs ? RowStats{0.f, 1.f} : row_stats(lrow, V, temperature, red);
+    auto wf = [&](int k) { return prow ? ldcg(prow + k) : prob_of(ldcg(lrow + k), temperature, st.mx, st.sum); };
     float* q = q_all + ((size_t)b * gamma + j) * V;
-    for (int k = threadIdx.x; k < V; k += SAMPLE_THREADS) q[k] = row[k];
+    const unsigned long long Z = row_mass(wf, [&](int k, float w) { stcg(q + k, w); }, V, rs, &sc);
+    row_pick(wf, V, Z, u[(size_t)b * gamma + j], rs, &sc, tok);
   }
   if (threadIdx.x == 0) seqs[b].st->d_ids[j] = tok;
 }
 
-// The rejection rule and the commit, one CTA per sequence (Sec. 2.1): rows [B][gamma+1][V] are the
-// target's probability rows (logit rows when greedy: only their arg-max is used), q_all
-// [B][gamma][V] the draft's.  Each sequence advances by its own accepted count.
-__global__ void __launch_bounds__(SAMPLE_THREADS) batch_verify_kernel(const BatchSeq* seqs, const float* rows,
-                                                                      const float* q_all, const float* u, int gamma,
-                                                                      int V, int greedy, int* n_acc, int* next) {
-  __shared__ SampleScratch sc;
+// The rejection rule and the commit, C CTAs per sequence (Sec. 2.1): the target's rows are logits
+// [B][gamma+1][V] with their statistics, or probability rows when truncated (greedy: only the arg-max of
+// the logits is used); q_all [B][gamma][V] the draft's.  Each sequence advances by its own count.
+__global__ void __launch_bounds__(ROW_THREADS) batch_verify_kernel(const BatchSeq* seqs, int C, const float* logits,
+                                                                   const RowStats* stats, const float* probs, const float* q_all,
+                                                                   const float* u, int gamma, int V, int greedy, float temperature,
+                                                                   int* n_acc, int* next) {
+  __shared__ RowScratch sc;
   __shared__ int s_ids[MAX_M];
   pdl_wait();
   pdl_trigger();
-  const int b = blockIdx.x;
+  const int b = blockIdx.x / C;
+  const RowSlice rs = row_slice(C);
   DevState* st = seqs[b].st;
   if (threadIdx.x < gamma) {
     const int x = st->d_ids[threadIdx.x];
     s_ids[threadIdx.x] = (unsigned)x < (unsigned)V ? x : 0;   // the embedding kernel has flagged it
   }
-  named_sync(1, SAMPLE_THREADS);
+  __syncthreads();
+  const size_t row0 = (size_t)b * (gamma + 1);
+  auto pv = [&](int j, int k) {
+    if (probs) return ldcg(probs + (row0 + j) * V + k);
+    const float l = ldcg(logits + (row0 + j) * V + k);
+    return greedy ? l : prob_of(l, temperature, stats[row0 + j].mx, stats[row0 + j].sum);
+  };
+  auto qv = [&](int j, int k) { return ldcg(q_all + ((size_t)b * gamma + j) * V + k); };
   int r, tok;
-  reject_rule_block(rows + (size_t)b * (gamma + 1) * V, q_all + (size_t)b * gamma * V, s_ids,
-                    u ? u + (size_t)b * (gamma + 1) : nullptr, gamma, V, greedy, &sc, r, tok);
-  if (threadIdx.x == 0) {
+  const bool mine = rule_rows(pv, qv, s_ids, u ? u + row0 : nullptr, gamma, V, greedy, rs, &sc, r, tok);
+  if (mine && threadIdx.x == 0) {
     st->n_acc = r;
     st->next = tok;
     st->n_text += r + 1;

@@ -74,8 +74,6 @@ struct ModelDev {
   float *apart, *aml;                 // attention partials [H][nsplit][8][dh], [H][nsplit][8][2]
   unsigned* head_cnt;                 // [H]
   float* stat_part;                   // [grid][8][4]: row max, row sum, argmax value, argmax index
-  unsigned long long* cdf_part;       // [grid][2]: integer mass of the CTA's vocabulary slice, (max weight, index);
-                                      // then [2]: accepted count r, (max, sum exp) of row r for the pick kernel
   const LayerDev* layers;
 };
 
@@ -1386,7 +1384,7 @@ __device__ void merge_stats(const float* stat_part, int G, int nrows, Ctrl* ctl,
   named_sync(1, CONSUMER_THREADS);
 }
 
-__device__ __noinline__ float prob_of(float logit, float temperature, float rmax, float rsum) {
+__device__ __forceinline__ float prob_of(float logit, float temperature, float rmax, float rsum) {
   return __fdiv_rn(expf(__fsub_rn(__fdiv_rn(logit, temperature), rmax)), rsum);
 }
 

@@ -34,8 +34,8 @@ __device__ __forceinline__ void commit_step(const StepArgs& a, DevState* st, int
 // Greedy decoding (Sec. 4 "Decoding"), run by CTA 0 after the row statistics are merged: a draft
 // token is accepted iff it is the argmax of the target's row; the next token is the argmax of the
 // first mismatching row, or of row gamma.  Rows r0..r0+gamma of `logits` are p_1..p_{gamma+1}.
-// (With sampling the forward kernel stops after the row statistics and the two sampling kernels
-// below finish the step.)
+// (With sampling the forward kernel stops after the row statistics and the sampling kernel below
+// finishes the step.)
 template <int M>
 __device__ void verify_greedy(const StepArgs& a, const ModelDev& md, DevState* st, Ctrl* ctl, int G, int r0,
                               int gamma, const int* ids /*gamma draft ids*/, int pending) {
@@ -288,26 +288,18 @@ __global__ void __launch_bounds__(CONSUMER_THREADS) wait_selftest_kernel(DevStat
 // Speculative sampling proper (Sec. 2.1 / Sec. 3; p = target, q = draft): accept x_j iff
 // u_j < min(1, p_j(x_j) / q_j(x_j)); the first rejected token is replaced by a draw from
 // max(0, p_r - q_r) / sum, and if none is rejected a bonus token is drawn from p_{gamma+1}.
-// The work that touches a whole vocabulary row is spread over the grid, in two small launches
-// behind the forward kernel (which has left the logits and the per-slice row statistics):
-//   sample_slices_kernel  every CTA merges the row statistics, repeats the (cheap, deterministic)
-//                         accept tests to find r, and reduces its contiguous vocabulary slice of
-//                         the weights the next token is drawn from to an integer mass; a draft
-//                         step also writes its slice of q_j = softmax(logits / T);
-//   sample_pick_kernel    one CTA finds the slice and the token, and commits the step.
-// They are separate kernels, not phases of the forward kernel, because that kernel's weight
-// streaming loop lost 1.5-2 % of its speed whenever this code was compiled into it.
+// The work that touches a whole vocabulary row runs on one cluster of CTAs in a small launch behind the
+// forward kernel (which has left the logits and the per-slice row statistics): every CTA merges the
+// statistics, makes the (independent) accept tests in parallel, reduces its vocabulary slice of the
+// weights to an integer mass -- a draft step also writes its slice of q_j = softmax(logits / T) --
+// and the CTA that holds the token commits the step.  It is a separate kernel, not a phase of the
+// forward kernel, because that kernel's weight streaming loop lost 1.5-2 % of its speed whenever this
+// code was compiled into it.
 
 struct SampleShared {
   float rowmax[MAX_M], rowsum[MAX_M];
   int arg[MAX_M];
-  SampleScratch sc;
-};
-
-struct SamplePlan {
-  int r0, gamma;  // first row and number of draft tokens
-  int r;          // accepted draft tokens = row the next token is drawn from
-  const float* u; // uniforms of this step: gamma accept tests, then the draw
+  RowScratch rows;
 };
 
 __device__ __forceinline__ const float* step_uniforms(const StepArgs& a, const DevState* st) {
@@ -315,85 +307,43 @@ __device__ __forceinline__ const float* step_uniforms(const StepArgs& a, const D
   return (a.mode == MODE_VERIFY && a.u_by_block) ? u + a.gamma : u;
 }
 
-// Every thread of every CTA computes the same plan (same inputs, same arithmetic).
-__device__ SamplePlan sample_plan(const StepArgs& a, const DevState* st, SampleShared* sh, int G) {
-  const int V = a.md.V;
-  SamplePlan pl;
-  pl.gamma = a.mode == MODE_VERIFY ? a.gamma : 0;
-  pl.r0 = a.mode == MODE_VERIFY ? 0 : a.sample_r0;
-  pl.u = step_uniforms(a, st);
-  merge_stats(a.md.stat_part, a.fwd_grid, pl.gamma + 1, nullptr, sh->rowmax, sh->rowsum, sh->arg);
-  pl.r = pl.gamma;
-  for (int j = 0; j < pl.gamma; ++j) {
-    int x = st->d_ids[j];
-    if ((unsigned)x >= (unsigned)V) x = 0;   // the forward kernel has flagged it; stay in bounds
-    const float p = prob_of(ldcg(a.logits + (size_t)(pl.r0 + j) * V + x), a.temperature, sh->rowmax[j], sh->rowsum[j]);
-    const float q = ldcg(a.q_in + (size_t)j * V + x);
-    if (!accept_test(pl.u[j], p, q)) { pl.r = j; break; }
-  }
-  return pl;
+// merge_stats by the first 8 warps of a CTA of ROW_THREADS
+__device__ __forceinline__ void merge_stats_rows(const StepArgs& a, int nrows, SampleShared* sh) {
+  if (threadIdx.x < CONSUMER_THREADS) merge_stats(a.md.stat_part, a.fwd_grid, nrows, nullptr, sh->rowmax, sh->rowsum, sh->arg);
+  __syncthreads();
 }
 
-// Calls f(weight function) with the weights of the row the next token is drawn from.
-template <class F>
-__device__ __forceinline__ void with_weights(const StepArgs& a, const SamplePlan& pl, const SampleShared* sh, F f) {
-  const int V = a.md.V;
-  const float* lrow = a.logits + (size_t)(pl.r0 + pl.r) * V;
-  const float mx = sh->rowmax[pl.r], sm = sh->rowsum[pl.r], T = a.temperature;
-  if (a.mode == MODE_DRAFT || pl.r == pl.gamma) {
-    f([=](int k) { return prob_of(ldcg(lrow + k), T, mx, sm); });
-  } else {
-    const float* qrow = a.q_in + (size_t)pl.r * V;
-    f([=](int k) { return fmaxf(0.0f, __fsub_rn(prob_of(ldcg(lrow + k), T, mx, sm), ldcg(qrow + k))); });
-  }
-}
-
-__global__ void __launch_bounds__(SAMPLE_THREADS) sample_slices_kernel(const __grid_constant__ StepArgs a) {
+__global__ void __launch_bounds__(ROW_THREADS) sample_step_kernel(const __grid_constant__ StepArgs a, int C) {
   __shared__ SampleShared sh;
-  const int cta = blockIdx.x, G = gridDim.x, V = a.md.V;
-  const SamplePlan pl = sample_plan(a, a.st, &sh, G);
-  if (cta == 0 && threadIdx.x == 0) {   // the plan travels to the pick kernel behind the slice masses
-    __stcg(a.md.cdf_part + 2 * G, (unsigned long long)pl.r);
-    __stcg(a.md.cdf_part + 2 * G + 1,
-           ((unsigned long long)__float_as_uint(sh.rowmax[pl.r]) << 32) | __float_as_uint(sh.rowsum[pl.r]));
-  }
-  with_weights(a, pl, &sh, [&](auto wf) {
-    if (a.mode == MODE_DRAFT) {   // this CTA's slice of q_j
-      float* qrow = a.q_out + (size_t)a.j * V;
-      const int VS = (V + G - 1) / G;
-      const int k0 = cta * VS, k1 = min(V, k0 + VS);
-      for (int k = k0 + threadIdx.x; k < k1; k += SAMPLE_THREADS) stcg(qrow + k, wf(k));
-    }
-    slice_mass(wf, V, cta, G, a.md.cdf_part, &sh.sc);
-  });
-}
-
-// One CTA; G = number of slices = the grid of the two kernels before it.
-__global__ void __launch_bounds__(SAMPLE_THREADS) sample_pick_kernel(const __grid_constant__ StepArgs a, int G) {
-  __shared__ SampleShared sh;
+  __shared__ int s_ids[MAX_M];
   DevState* st = a.st;
-  SamplePlan pl;   // r and the statistics of row r as the slices kernel found them
-  pl.gamma = a.mode == MODE_VERIFY ? a.gamma : 0;
-  pl.r0 = a.mode == MODE_VERIFY ? 0 : a.sample_r0;
-  pl.u = step_uniforms(a, st);
-  pl.r = (int)__ldcg(a.md.cdf_part + 2 * G);
-  if (pl.r < 0 || pl.r > pl.gamma) pl.r = pl.gamma;
-  if (threadIdx.x == 0) {
-    const unsigned long long ms = __ldcg(a.md.cdf_part + 2 * G + 1);
-    sh.rowmax[pl.r] = __uint_as_float((unsigned)(ms >> 32));
-    sh.rowsum[pl.r] = __uint_as_float((unsigned)ms);
+  const RowSlice rs = row_slice(C);
+  const int V = a.md.V, gamma = a.mode == MODE_VERIFY ? a.gamma : 0, r0 = a.mode == MODE_VERIFY ? 0 : a.sample_r0;
+  const float* u = step_uniforms(a, st);
+  if (threadIdx.x < gamma) {
+    const int x = st->d_ids[threadIdx.x];
+    s_ids[threadIdx.x] = (unsigned)x < (unsigned)V ? x : 0;   // the forward kernel has flagged it; stay in bounds
   }
-  named_sync(1, SAMPLE_THREADS);
-  int tok = 0;
-  with_weights(a, pl, &sh, [&](auto wf) {
-    tok = pick_from_slices(wf, a.md.V, G, a.md.cdf_part, a.mode == MODE_DRAFT ? pl.u[a.j] : pl.u[pl.gamma], &sh.sc);
-  });
-  if (threadIdx.x == 0) {
+  merge_stats_rows(a, gamma + 1, &sh);
+  const float T = a.temperature;
+  int r = 0, tok = 0;
+  bool mine;
+  if (a.mode == MODE_DRAFT) {
+    const float* lrow = a.logits + (size_t)r0 * V;
+    float* qrow = a.q_out + (size_t)a.j * V;
+    auto wf = [&](int k) { return prob_of(ldcg(lrow + k), T, sh.rowmax[0], sh.rowsum[0]); };
+    const unsigned long long Z = row_mass(wf, [&](int k, float w) { stcg(qrow + k, w); }, V, rs, &sh.rows);
+    mine = row_pick(wf, V, Z, u[a.j], rs, &sh.rows, tok);
+  } else {
+    mine = rule_rows([&](int j, int k) { return prob_of(ldcg(a.logits + (size_t)(r0 + j) * V + k), T, sh.rowmax[j], sh.rowsum[j]); },
+                     [&](int j, int k) { return ldcg(a.q_in + (size_t)j * V + k); }, s_ids, u, gamma, V, 0, rs, &sh.rows, r, tok);
+  }
+  if (mine && threadIdx.x == 0) {
     if (a.mode == MODE_DRAFT) {
       st->d_ids[a.j] = tok;
       st->t_draft1 = globaltimer();
     } else {
-      commit_step(a, st, pl.r, tok, st->d_ids, st->pending);
+      commit_step(a, st, r, tok, st->d_ids, st->pending);
       if (a.mode == MODE_VERIFY) st->t_verify1 = globaltimer();
     }
   }
@@ -406,11 +356,13 @@ __global__ void __launch_bounds__(SAMPLE_THREADS) sample_pick_kernel(const __gri
 //   prob_rows_kernel    every CTA merges the row statistics and writes its vocabulary slice of
 //                       softmax(logits / T) for the rows the step needs -> prow [rows][V];
 //   (truncate_rows_kernel in place on prow)
-//   sample_rows_kernel  one CTA: draft step -> x_j drawn from the truncated row, which is also
+//   sample_rows_kernel  one cluster: draft step -> x_j drawn from the truncated row, which is also
 //                       stored as q_j; verify step -> the rule on (prow, q_in), commit; prefill ->
 //                       the first token drawn from the truncated row.
 
-__global__ void __launch_bounds__(SAMPLE_THREADS) prob_rows_kernel(const __grid_constant__ StepArgs a, float* prow) {
+constexpr int PROB_THREADS = 256;
+
+__global__ void __launch_bounds__(PROB_THREADS) prob_rows_kernel(const __grid_constant__ StepArgs a, float* prow) {
   __shared__ SampleShared sh;
   const int cta = blockIdx.x, G = gridDim.x, V = a.md.V;
   const int nrows = a.stat_n, r0 = a.stat_r0;
@@ -421,38 +373,41 @@ __global__ void __launch_bounds__(SAMPLE_THREADS) prob_rows_kernel(const __grid_
   for (int r = 0; r < nrows; ++r) {
     const float* lrow = a.logits + (size_t)(r0 + r) * V;
     const float mx = sh.rowmax[r], sm = sh.rowsum[r];
-    for (int k = k0 + threadIdx.x; k < k1; k += SAMPLE_THREADS)
+    for (int k = k0 + threadIdx.x; k < k1; k += PROB_THREADS)
       stcg(prow + (size_t)r * V + k, prob_of(ldcg(lrow + k), a.temperature, mx, sm));
   }
 }
 
-__global__ void __launch_bounds__(SAMPLE_THREADS) sample_rows_kernel(const __grid_constant__ StepArgs a,
-                                                                     const float* prow) {
-  __shared__ SampleScratch sc;
+__global__ void __launch_bounds__(ROW_THREADS) sample_rows_kernel(const __grid_constant__ StepArgs a, int C, const float* prow) {
+  __shared__ RowScratch sc;
   __shared__ int s_ids[MAX_M];
   DevState* st = a.st;
+  const RowSlice rs = row_slice(C);
   const int V = a.md.V;
   const float* u = step_uniforms(a, st);
+  int r = 0, tok = 0;
+  bool mine;
   if (a.mode == MODE_VERIFY) {
     if (threadIdx.x < a.gamma) {
       const int x = st->d_ids[threadIdx.x];
       s_ids[threadIdx.x] = (unsigned)x < (unsigned)V ? x : 0;   // the forward kernel has flagged it
     }
-    named_sync(1, SAMPLE_THREADS);
-    int r, tok;
-    reject_rule_block(prow, a.q_in, s_ids, u, a.gamma, V, 0, &sc, r, tok);
-    if (threadIdx.x == 0) {
-      commit_step(a, st, r, tok, st->d_ids, st->pending);
-      st->t_verify1 = globaltimer();
-    }
+    __syncthreads();
+    mine = rule_rows([&](int j, int k) { return ldcg(prow + (size_t)j * V + k); },
+                     [&](int j, int k) { return ldcg(a.q_in + (size_t)j * V + k); }, s_ids, u, a.gamma, V, 0, rs, &sc, r, tok);
   } else {
-    const int tok = block_sample([&](int k) { return ldcg(prow + k); }, V, a.mode == MODE_DRAFT ? u[a.j] : u[0], &sc);
+    auto wf = [&](int k) { return ldcg(prow + k); };
+    float* qrow = a.mode == MODE_DRAFT ? a.q_out + (size_t)a.j * V : nullptr;
+    const unsigned long long Z = row_mass(wf, [&](int k, float w) { if (qrow) stcg(qrow + k, w); }, V, rs, &sc);
+    mine = row_pick(wf, V, Z, a.mode == MODE_DRAFT ? u[a.j] : u[0], rs, &sc, tok);
+  }
+  if (mine && threadIdx.x == 0) {
     if (a.mode == MODE_DRAFT) {
-      float* qrow = a.q_out + (size_t)a.j * V;
-      for (int k = threadIdx.x; k < V; k += SAMPLE_THREADS) stcg(qrow + k, ldcg(prow + k));
-      if (threadIdx.x == 0) { st->d_ids[a.j] = tok; st->t_draft1 = globaltimer(); }
-    } else if (threadIdx.x == 0) {
-      commit_step(a, st, 0, tok, st->d_ids, st->pending);
+      st->d_ids[a.j] = tok;
+      st->t_draft1 = globaltimer();
+    } else {
+      commit_step(a, st, r, tok, st->d_ids, st->pending);
+      if (a.mode == MODE_VERIFY) st->t_verify1 = globaltimer();
     }
   }
 }

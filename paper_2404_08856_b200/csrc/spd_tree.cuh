@@ -26,61 +26,69 @@ namespace spd {
 // its probability row prow[k] is stored as Q[node] and every child c is drawn from it with u[c-1]
 // (independent draws, repeats allowed).  Greedy: the children are the most probable tokens of the
 // row, in order, lower index first among equal logits.
-__global__ void __launch_bounds__(SAMPLE_THREADS) tree_draw_kernel(const __grid_constant__ StepArgs a,
-                                                                   const TreeShape shape, const float* prow) {
-  __shared__ SampleScratch sc;
+// C CTAs per row.  truncated: prow holds the (truncated) probability rows; else they are computed here
+// from the logits and the row statistics.
+__global__ void __launch_bounds__(ROW_THREADS) tree_draw_kernel(const __grid_constant__ StepArgs a, const TreeShape shape, int C,
+                                                                const float* prow, int truncated) {
+  __shared__ SampleShared sh;
   __shared__ int taken[MAX_M];
   DevState* st = a.st;
-  const int V = a.md.V;
+  const int V = a.md.V, k = blockIdx.x / C;
+  const RowSlice rs = row_slice(C);
   const float* u = step_uniforms(a, st);
-  for (int k = 0; k < a.stat_n; ++k) {
-    const int node = a.geo.slot[a.stat_r0 + k];
-    const float* lrow = a.logits + (size_t)(a.stat_r0 + k) * V;
+  const int node = a.geo.slot[a.stat_r0 + k];
+  const float* lrow = a.logits + (size_t)(a.stat_r0 + k) * V;
+  if (!a.greedy) {
+    if (!truncated) merge_stats_rows(a, a.stat_n, &sh);
     const float* row = prow + (size_t)k * V;
-    if (!a.greedy) {
-      float* qrow = a.q_out + (size_t)node * V;
-      for (int i = threadIdx.x; i < V; i += SAMPLE_THREADS) stcg(qrow + i, ldcg(row + i));
-    }
-    int n_taken = 0;
+    const float mx = sh.rowmax[k], sm = sh.rowsum[k];
+    auto wf = [&](int i) { return truncated ? ldcg(row + i) : prob_of(ldcg(lrow + i), a.temperature, mx, sm); };
+    float* qrow = a.q_out + (size_t)node * V;
+    const unsigned long long Z = row_mass(wf, [&](int i, float w) { stcg(qrow + i, w); }, V, rs, &sh.rows);
     for (int c = 1; c <= shape.n; ++c) {
       if (shape.parent[c] != node) continue;
       int tok;
-      if (a.greedy) {
-        const int nt = n_taken;
-        tok = block_argmax([&](int i) {
-          bool used = false;
-          for (int t = 0; t < nt; ++t) used |= taken[t] == i;
-          return used ? -INFINITY : ldcg(lrow + i);
-        }, V, &sc);
-        if (threadIdx.x == 0) taken[n_taken] = tok;
-        ++n_taken;
-        named_sync(1, SAMPLE_THREADS);
-      } else {
-        tok = block_sample([&](int i) { return ldcg(row + i); }, V, u[c - 1], &sc);
+      if (row_pick(wf, V, Z, u[c - 1], rs, &sh.rows, tok) && threadIdx.x == 0) st->d_ids[c - 1] = tok;
+    }
+  } else {
+    int n_taken = 0;
+    for (int c = 1; c <= shape.n; ++c) {
+      if (shape.parent[c] != node) continue;
+      const int nt = n_taken;
+      rows_argmax([&](int, int i) {
+        bool used = false;
+        for (int t = 0; t < nt; ++t) used |= taken[t] == i;
+        return used ? -INFINITY : ldcg(lrow + i);
+      }, 1, V, rs, &sh.rows);
+      const int tok = sh.rows.arg[0];
+      if (threadIdx.x == 0) {
+        taken[n_taken] = tok;
+        if (rs.rank == 0) st->d_ids[c - 1] = tok;
       }
-      if (threadIdx.x == 0) st->d_ids[c - 1] = tok;
+      ++n_taken;
+      cluster_sync_all_threads();   // `taken` and the exchange buffers are used again
     }
   }
-  if (threadIdx.x == 0) st->t_draft1 = globaltimer();
+  if (blockIdx.x == 0 && threadIdx.x == 0) st->t_draft1 = globaltimer();
 }
 
 // ---- target side: the rule on the rows of one verify launch, then the commit
 // prow [n+1][V] target probability rows (unused when greedy: the arg-max of each row comes from the
 // row statistics), q_in [n+1][V] draft rows, cur [V] scratch for a renormalised residual.
-__global__ void __launch_bounds__(SAMPLE_THREADS) tree_verify_kernel(const __grid_constant__ StepArgs a,
-                                                                     const TreeShape shape, const float* prow,
-                                                                     float* cur_buf) {
+__global__ void __launch_bounds__(ROW_THREADS) tree_verify_kernel(const __grid_constant__ StepArgs a, const TreeShape shape,
+                                                                  const float* prow, float* cur_buf) {
   __shared__ SampleShared sh;
   __shared__ int s_ids[MAX_M], s_path_ids[MAX_M], s_path[MAX_M];
   DevState* st = a.st;
   const int V = a.md.V, n = shape.n, tid = threadIdx.x;
+  const RowSlice rs{0, 1};      // one CTA: the walk is a chain of decisions
   const float* u = step_uniforms(a, st);
   if (tid < n) {
     const int x = st->d_ids[tid];
     s_ids[tid] = (unsigned)x < (unsigned)V ? x : 0;   // the forward kernel has flagged it
   }
-  if (a.greedy) merge_stats(a.md.stat_part, a.fwd_grid, n + 1, nullptr, sh.rowmax, sh.rowsum, sh.arg);
-  named_sync(1, SAMPLE_THREADS);
+  if (a.greedy) merge_stats_rows(a, n + 1, &sh);
+  __syncthreads();
   int node = 0, plen = 0, tok = 0;
   while (true) {
     const float* cur = prow + (size_t)node * V;        // P[node]; becomes cur_buf after a rejection
@@ -99,22 +107,16 @@ __global__ void __launch_bounds__(SAMPLE_THREADS) tree_verify_kernel(const __gri
       if (accept_test(u[c - 1], ldcg(cur + x), ldcg(qrow + x))) { took = c; break; }
       if (c != last_child) {
         // cur <- max(0, cur - q) / sum, the sum taken over integer masses
-        unsigned long long z = 0;
-        for (int i = tid; i < V; i += SAMPLE_THREADS) z += to_fixed(fmaxf(0.0f, __fsub_rn(ldcg(cur + i), ldcg(qrow + i))));
-#pragma unroll
-        for (int o = 16; o; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-        named_sync(1, SAMPLE_THREADS);
-        if ((tid & 31) == 0) sh.sc.wsum[tid >> 5] = z;
-        named_sync(1, SAMPLE_THREADS);
-        unsigned long long Z = 0;
-#pragma unroll
-        for (int w = 0; w < 8; ++w) Z += sh.sc.wsum[w];
+        const float* c0 = cur;
+        auto left = [&](int i) { return fmaxf(0.0f, __fsub_rn(ldcg(c0 + i), ldcg(qrow + i))); };
+        const unsigned long long Z = row_mass(left, [](int, float) {}, V, rs, &sh.rows);
         const float S = __fmul_rn(__ull2float_rn(Z), 2.3283064365386963e-10f);
-        for (int i = tid; i < V; i += SAMPLE_THREADS) {
-          const float w = fmaxf(0.0f, __fsub_rn(ldcg(cur + i), ldcg(qrow + i)));
+#pragma unroll 8
+        for (int i = tid; i < V; i += ROW_THREADS) {   // (in place after the first rejection: element by element)
+          const float w = left(i);
           stcg(cur_buf + i, Z ? __fdiv_rn(w, S) : w);
         }
-        named_sync(1, SAMPLE_THREADS);
+        __syncthreads();
         cur = cur_buf;
       } else {
         residual = true;
@@ -123,17 +125,17 @@ __global__ void __launch_bounds__(SAMPLE_THREADS) tree_verify_kernel(const __gri
     if (took < 0) {
       if (a.greedy) tok = sh.arg[node];
       else if (residual)
-        tok = block_sample([&](int i) { return fmaxf(0.0f, __fsub_rn(ldcg(cur + i), ldcg(qrow + i))); }, V, u[n], &sh.sc);
+        row_sample([&](int i) { return fmaxf(0.0f, __fsub_rn(ldcg(cur + i), ldcg(qrow + i))); }, V, u[n], rs, &sh.rows, tok);
       else
-        tok = block_sample([&](int i) { return ldcg(cur + i); }, V, u[n], &sh.sc);
+        row_sample([&](int i) { return ldcg(cur + i); }, V, u[n], rs, &sh.rows, tok);
       break;
     }
     if (tid == 0) { s_path[plen] = took; s_path_ids[plen] = s_ids[took - 1]; }
     ++plen;
     node = took;
-    named_sync(1, SAMPLE_THREADS);
+    __syncthreads();
   }
-  named_sync(1, SAMPLE_THREADS);
+  __syncthreads();
   if (tid == 0) {
     for (int j = 0; j < plen; ++j) st->path[j] = s_path[j];
     commit_step(a, st, plen, tok, s_path_ids, st->pending);
