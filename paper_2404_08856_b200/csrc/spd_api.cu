@@ -1482,6 +1482,8 @@ struct spd_batch {
   ModelDev *mds_t = nullptr, *mds_d = nullptr;
   int *rowslot = nullptr, *origins = nullptr, *out_acc = nullptr, *out_next = nullptr;
   RowStats* stats = nullptr;    // (max, sum exp) of the rows of a verify step
+  float *part_o = nullptr, *part_ml = nullptr;   // attention partials of the KV splits
+  unsigned* attn_cnt = nullptr;
   float *X = nullptr, *logits = nullptr, *probs = nullptr, *q_all = nullptr, *u_draft = nullptr, *u_verify = nullptr;
   int drafted_gamma = -1;
   int last_rows = 0;
@@ -1509,34 +1511,22 @@ spd_status balloc(spd_batch* bt, T** p, size_t n) {
   return SPD_OK;
 }
 
-constexpr int BATCH_ATTN_SCRATCH = 100 * 1024;   // two CTAs per SM: 16 warps hide each other's dependency stalls
-
-template <int M>
-spd_status launch_batch_attn(spd_ctx* ctx, const ModelDev* mds, const int* origins, int B, int layer, int chain0,
-                             int max_split, __nv_bfloat16* o_hi, __nv_bfloat16* o_lo) {
+template <int DH>
+spd_status launch_batch_attn(spd_ctx* ctx, const BatchAttnArgs& a) {
   static bool attr[MAX_DEV];
-  const size_t smem = CTRL_BYTES + BATCH_ATTN_SCRATCH;
   if (!attr[ctx->device]) {
-    CU(cudaFuncSetAttribute((const void*)batch_attn_kernel<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CU(cudaFuncSetAttribute((const void*)batch_attn_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, BA_SMEM));
     attr[ctx->device] = true;
   }
-  CU(launch_dependent(batch_attn_kernel<M>, dim3(2 * ctx->n_sm), dim3(CONSUMER_THREADS), smem, ctx->stream, mds, origins, B, layer,
-                      chain0, BATCH_ATTN_SCRATCH, max_split, o_hi, o_lo));
+  CU(launch_dependent(batch_attn_kernel<DH>, dim3(ctx->n_sm), dim3(BA_WARPS * 32), BA_SMEM, ctx->stream, a));
   return SPD_OK;
 }
 
-spd_status batch_attn(spd_ctx* ctx, int M, const ModelDev* mds, const int* origins, int B, int layer, int chain0,
-                      int max_split, __nv_bfloat16* o_hi, __nv_bfloat16* o_lo) {
-  switch (M) {
-    case 1: return launch_batch_attn<1>(ctx, mds, origins, B, layer, chain0, max_split, o_hi, o_lo);
-    case 2: return launch_batch_attn<2>(ctx, mds, origins, B, layer, chain0, max_split, o_hi, o_lo);
-    case 3: return launch_batch_attn<3>(ctx, mds, origins, B, layer, chain0, max_split, o_hi, o_lo);
-    case 4: return launch_batch_attn<4>(ctx, mds, origins, B, layer, chain0, max_split, o_hi, o_lo);
-    case 5: return launch_batch_attn<5>(ctx, mds, origins, B, layer, chain0, max_split, o_hi, o_lo);
-    case 6: return launch_batch_attn<6>(ctx, mds, origins, B, layer, chain0, max_split, o_hi, o_lo);
-    case 7: return launch_batch_attn<7>(ctx, mds, origins, B, layer, chain0, max_split, o_hi, o_lo);
-    default: return launch_batch_attn<8>(ctx, mds, origins, B, layer, chain0, max_split, o_hi, o_lo);
-  }
+// KV splits per head: as many (sequence, head, split) units as there are warps, so that all of them run at
+// once and end together.
+int batch_splits(int n_sm, int B, int H) {
+  const int s = n_sm * BA_WARPS / (B * H);
+  return s < 1 ? 1 : s;
 }
 
 // Dense forward of the B x M rows of a batched step through every layer and the LM head of one
@@ -1554,13 +1544,11 @@ spd_status batch_forward(spd_batch* bt, bool draft, int M, int j) {
   const ModelDev* mds = draft ? bt->mds_d : bt->mds_t;
   CU(launch_dependent(batch_embed_kernel, dim3(R), dim3(128), 0, cs, bt->seqs_dev, B, M, draft ? 1 : 0, j, mh.md.embed, d, V, X,
                       bt->rowslot, bt->origins, &ctx->st->err));
-  // KV splits per head: about two (sequence, head, split) units per SM, never more than a single
-  // sequence would use.  (Choosing the split count for an even division of the units over the CTAs
-  // was measured slower: 16 x 32 heads in 2 splits balance better than in 1 but pay for the merges,
-  // batched verify 12.6 -> 13.3 ms.)
-  int attn_split = (2 * ctx->n_sm + B * H - 1) / (B * H);
-  if (attn_split > mh.md.nsplit) attn_split = mh.md.nsplit;
-  if (attn_split < 1) attn_split = 1;
+  BatchAttnArgs at{};
+  at.mds = mds; at.origins = bt->origins; at.B = B; at.H = H; at.d = d; at.M = M;
+  at.chain0 = draft ? j - 1 : 0; at.splits = batch_splits(ctx->n_sm, B, H); at.scale = mh.md.scale;
+  at.part_o = bt->part_o; at.part_ml = bt->part_ml; at.cnt = bt->attn_cnt;
+  at.o_hi = pf.h_hi; at.o_lo = pf.h_lo;   // the operand of the output projection
   // Where a projection is cut into K slices, the kernel that reads its result adds the slices up
   // (in slice order): the rotary / cache-append kernel for QKV, the fused residual + RMSNorm + split
   // kernel for the output and down projections.
@@ -1574,8 +1562,8 @@ spd_status batch_forward(spd_batch* bt, bool draft, int M, int j) {
     if ((s = ug_gemm(ctx, pf.h_hi, pf.h_lo, R, d, w.wqkv, 3 * d, UG_F32, pf.wide, nullptr, nullptr, 3 * d, UG_SLICES_MAX, &sl))) return s;
     CU(launch_dependent(batch_rope_append_kernel, dim3(rope_blocks), dim3(128), 0, cs, pf.wide, sl, R, M, d, dh, bt->rowslot,
                         mh.md.rope_cos, mh.md.rope_sin, mds, l));
-    // (the attention kernel leaves its rows as the hi/lo operand of the output projection)
-    if ((s = batch_attn(ctx, M, mds, bt->origins, B, l, draft ? j - 1 : 0, attn_split, pf.h_hi, pf.h_lo))) return s;
+    at.layer = l;
+    if ((s = dh == 128 ? launch_batch_attn<128>(ctx, at) : launch_batch_attn<64>(ctx, at))) return s;
     if ((s = ug_gemm(ctx, pf.h_hi, pf.h_lo, R, d, w.wo, d, UG_F32, pf.wide, nullptr, nullptr, d, UG_SLICES_MAX, &sl))) return s;
     CU(launch_dependent(resid_rms_split_kernel, dim3(R), dim3(256), 0, cs, X, pf.wide, sl, xs, w.ffn_norm, mh.cfg.rms_eps, d, pf.h_hi,
                         pf.h_lo));
@@ -1693,6 +1681,7 @@ spd_status spd_batch_create(spd_ctx* const* seqs, int B, spd_batch** out) {
   bt->seqs.assign(seqs, seqs + B);
   const int V = ctx->cfg.target.vocab;
   const size_t dmax = ctx->cfg.target.d_model > ctx->cfg.draft.d_model ? ctx->cfg.target.d_model : ctx->cfg.draft.d_model;
+  size_t po = 0, pu = 0, ph = 0;
   spd_status s = SPD_OK;
   if (!s) s = balloc(bt, &bt->seqs_dev, (size_t)B);
   if (!s) s = balloc(bt, &bt->mds_t, (size_t)B);
@@ -1708,6 +1697,15 @@ spd_status spd_batch_create(spd_ctx* const* seqs, int B, spd_batch** out) {
   if (!s) s = balloc(bt, &bt->q_all, (size_t)B * gm * V);
   if (!s) s = balloc(bt, &bt->u_draft, (size_t)B * MAX_M);
   if (!s) s = balloc(bt, &bt->u_verify, (size_t)B * MAX_M);
+  for (const spd_model_cfg* c : {&ctx->cfg.target, &ctx->cfg.draft}) {   // attention partials: the larger model's
+    const size_t u = (size_t)B * c->n_heads * batch_splits(ctx->n_sm, B, c->n_heads), dh = c->d_model / c->n_heads;
+    if (u * dh > po) po = u * dh;
+    if (u > pu) pu = u;
+    if ((size_t)B * c->n_heads > ph) ph = (size_t)B * c->n_heads;
+  }
+  if (!s) s = balloc(bt, &bt->part_o, po * 8);
+  if (!s) s = balloc(bt, &bt->part_ml, pu * 16);
+  if (!s) s = balloc(bt, &bt->attn_cnt, ph);
   if (!s && ctx->truncate &&
       cudaFuncSetAttribute((const void*)truncate_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)((size_t)V * sizeof(float))) != cudaSuccess)
@@ -1752,7 +1750,8 @@ spd_status spd_batch_draft(spd_batch* bt, int gamma, const float* uniforms, int3
       if ((r = batch_forward(bt, true, 2, j))) return r;
       // (each sequence's first row only refreshes the cache: nothing is drawn from it)
       if (ctx->truncate && (r = batch_probs(bt, B, 1, 2))) return r;
-      CU(launch_rows(batch_draft_sample_kernel, B, 1, ROW_THREADS, ctx->stream, true, bt->seqs_dev, bt->logits,
+      const int C = row_ctas(ctx->n_sm, B, V);
+      CU(launch_rows(batch_draft_sample_kernel, B, C, ROW_THREADS, ctx->stream, true, bt->seqs_dev, C, bt->logits,
                      ctx->truncate ? bt->probs : nullptr, V, gamma, j, ctx->cfg.greedy, ctx->cfg.temperature, bt->u_draft, bt->q_all));
       return SPD_OK;
     };

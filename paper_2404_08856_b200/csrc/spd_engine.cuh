@@ -1007,26 +1007,14 @@ __device__ __forceinline__ void split_frag(float2 xa, float2 xb, uint32_t& h0, u
   l1 = pack_bf16(xb.x - bf16lo(h1), xb.y - bf16hi(h1));
 }
 
-// Piece i of a K/V tile -> (row, 16-byte piece of the row).  The long units of the batched kernel
-// (SHIFT) use the fact that a row has a power-of-two number of pieces; the decode kernel keeps
-// the division (its instruction stream is left exactly as it was measured).
-template <bool SHIFT>
-__device__ __forceinline__ void piece_of(int i, int cpr, int csh, int& r, int& cc) {
-  if constexpr (SHIFT) { r = i >> csh; cc = i & (cpr - 1); }
-  else { r = i / cpr; cc = i - r * cpr; }
-}
-
 // bf16 KV cache: the same unit / split / merge scheme as attn_phase, with both products on
 // the tensor cores.  Scores: D[16 positions x 8 queries] = K tile (A, ldmatrix) x q^T (B,
 // fp32 q split into bf16 hi + lo).  Output: D[16 dims x 8 queries] = V^T (A, transposing
 // ldmatrix) x P^T (B, fp32 probabilities split the same way); warp w owns dims 16w..16w+15,
 // so no cross-warp reduction is needed.  Tile rows are 16-byte-chunk swizzled by position.
-// PIPE (the batched kernel, where a unit spans several sub-chunks): two K/V tile buffers, the
-// next sub-chunk's rows are requested before the current one is computed; with o_hi / o_lo the
-// head's output rows [M][d] also leave as bf16 hi + lo (the next GEMM's operand).
-template <int M, bool PIPE = false>
+template <int M>
 __device__ void attn_phase_mma(const ModelDev& md, int layer, int origin, int nslots, int cta, int G, char* xs,
-                               int xbytes, Ctrl* ctl, __nv_bfloat16* o_hi = nullptr, __nv_bfloat16* o_lo = nullptr) {
+                               int xbytes, Ctrl* ctl) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int H = md.H, dh = md.dh, d = md.d;
   const int len = origin + nslots;
@@ -1037,36 +1025,23 @@ __device__ void attn_phase_mma(const ModelDev& md, int layer, int origin, int ns
   const int qst = dh + 8;                                    // padded fp32 row of q
   const char* Kl = static_cast<const char*>(md.kcache) + (size_t)layer * md.max_seq * d * 2;
   const char* Vl = static_cast<const char*>(md.vcache) + (size_t)layer * md.max_seq * d * 2;
-  // scratch: q [M][dh+8] fp32 | NB x (K tile [SC][rowb] | V tile [SC][rowb]) | S [M][SC+8] fp32
-  // PIPE also keeps q and the probabilities as packed bf16 (hi, lo) pairs -- the B fragments of the
-  // MMAs as they are -- so that the fp32 -> hi/lo split is done once per unit / per probability
-  // instead of once per use: + Qh | Ql [M][dh/2+4] words behind q, + Ph | Pl [M][SC/2+4] words behind S
-  constexpr int NB = PIPE ? 2 : 1;
-  const int qw = (dh >> 1) + 4;                              // words per packed q row
-  const int qpk = PIPE ? 2 * M * qw * 4 : 0;
-  int SC = ((xbytes - M * qst * 4 - qpk - M * 8 * 4 - (PIPE ? M * 8 * 4 : 0)) / (2 * NB * rowb + M * (PIPE ? 8 : 4))) & ~15;
+  // scratch: q [M][dh+8] fp32 | K tile [SC][rowb] | V tile [SC][rowb] | S [M][SC+8] fp32
+  int SC = ((xbytes - M * qst * 4 - M * 8 * 4) / (2 * rowb + M * 4)) & ~15;
   {  // equal sub-chunks instead of full ones plus a sliver
     const int nsub = (Lc + SC - 1) / SC;
     SC = min(SC, (((Lc + nsub - 1) / nsub) + 15) & ~15);
   }
-  const int sst = SC + 8, pw = (SC >> 1) + 4;                // fp32 row of S, words per packed probability row
+  const int sst = SC + 8;                                    // fp32 row of S
   float* qs = reinterpret_cast<float*>(xs);
-  uint32_t* Qh = reinterpret_cast<uint32_t*>(xs + M * qst * 4);
-  uint32_t* Ql = Qh + M * qw;
-  char* const Kt0 = xs + M * qst * 4 + qpk;
+  char* const Kt = xs + M * qst * 4;
   const size_t tileb = (size_t)SC * rowb;
-  float* S = reinterpret_cast<float*>(Kt0 + 2 * NB * tileb);
-  uint32_t* Ph = reinterpret_cast<uint32_t*>(S + M * sst);
-  uint32_t* Pl = Ph + M * pw;
-  // request rows [c0, c0 + n) of the head's K and V into tile buffer `buf`
-  auto request = [&](int h, int c0, int n, int buf) {
-    char* Kt = Kt0 + (size_t)buf * 2 * tileb;
-    char* Vt = Kt + tileb;
+  char* const Vt = Kt + tileb;
+  float* S = reinterpret_cast<float*>(Kt + 2 * tileb);
+  // request rows [c0, c0 + n) of the head's K and V
+  auto request = [&](int h, int c0, int n) {
     const int n16 = (n + 15) & ~15;
-    const int csh = 31 - __clz(cpr);     // 16-byte pieces per row: a power of two
     for (int i = tid; i < n16 * cpr; i += CONSUMER_THREADS) {
-      int r, cc;
-      piece_of<PIPE>(i, cpr, csh, r, cc);
+      const int r = i / cpr, cc = i - r * cpr;
       const int dst = r * rowb + ((cc ^ (r & 7)) << 4);
       if (r < n) {
         const size_t g = (((size_t)h * md.max_seq + c0 + r) * dh) * 2 + (size_t)cc * 16;
@@ -1090,56 +1065,23 @@ __device__ void attn_phase_mma(const ModelDev& md, int layer, int origin, int ns
     }
     if (tid < M) { ctl->rowmax[tid] = -INFINITY; ctl->rowsum[tid] = 0.f; }
     float oacc[4] = {0.f, 0.f, 0.f, 0.f};
-    int buf = 0;
-    if (PIPE) request(h, p0, min(SC, p1 - p0), 0);
     for (int c0 = p0; c0 < p1; c0 += SC) {
       const int n = min(SC, p1 - c0), n16 = (n + 15) & ~15;
-      if (PIPE) {
-        const int c1 = c0 + SC;
-        if (c1 < p1) {
-          request(h, c1, min(SC, p1 - c1), buf ^ 1);
-          asm volatile("cp.async.wait_group 1;" ::: "memory");
-        } else {
-          asm volatile("cp.async.wait_group 0;" ::: "memory");
-        }
-      } else {
-        request(h, c0, n, 0);
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-      }
-      char* Kt = Kt0 + (size_t)buf * 2 * tileb;
-      char* Vt = Kt + tileb;
+      request(h, c0, n);
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
       named_sync(1, CONSUMER_THREADS);
-      if constexpr (PIPE) {
-        if (c0 == p0) {   // q has arrived with the first sub-chunk: split it once for the whole unit
-          for (int i = tid; i < M * (dh >> 1); i += CONSUMER_THREADS) {
-            const int m = i / (dh >> 1), j = i - m * (dh >> 1);
-            const float2 x = *reinterpret_cast<const float2*>(qs + m * qst + 2 * j);
-            const uint32_t hq = pack_bf16(x.x, x.y);
-            Qh[m * qw + j] = hq;
-            Ql[m * qw + j] = pack_bf16(x.x - bf16lo(hq), x.y - bf16hi(hq));
-          }
-          named_sync(1, CONSUMER_THREADS);
-        }
-      }
       // ---- scores: warp takes 16-position groups
       for (int gp = warp; gp * 16 < n; gp += 8) {
         float dsc[4] = {0.f, 0.f, 0.f, 0.f};
         for (int kd = 0; kd < nkd; ++kd) {
           uint32_t b0 = 0, b1 = 0, b2 = 0, b3 = 0;
-          if constexpr (PIPE) {
-            if (gq < M) {
-              const int w = gq * qw + kd * 8 + tq;
-              b0 = Qh[w]; b1 = Qh[w + 4]; b2 = Ql[w]; b3 = Ql[w + 4];
-            }
-          } else {
-            float2 xa = make_float2(0.f, 0.f), xb = make_float2(0.f, 0.f);
-            if (gq < M) {
-              const float* qr = qs + gq * qst + kd * 16 + 2 * tq;
-              xa = *reinterpret_cast<const float2*>(qr);
-              xb = *reinterpret_cast<const float2*>(qr + 8);
-            }
-            split_frag(xa, xb, b0, b1, b2, b3);
+          float2 xa = make_float2(0.f, 0.f), xb = make_float2(0.f, 0.f);
+          if (gq < M) {
+            const float* qr = qs + gq * qst + kd * 16 + 2 * tq;
+            xa = *reinterpret_cast<const float2*>(qr);
+            xb = *reinterpret_cast<const float2*>(qr + 8);
           }
+          split_frag(xa, xb, b0, b1, b2, b3);
           const int r = gp * 16 + (mat & 1) * 8 + rr;
           const int ch = (kd * 2 + (mat >> 1)) ^ (r & 7);
           uint32_t a0, a1, a2, a3;
@@ -1169,21 +1111,10 @@ __device__ void attn_phase_mma(const ModelDev& md, int layer, int origin, int ns
         const float old = ctl->rowmax[warp];
         const float nm = fmaxf(old, mx);
         float sum = 0.f;
-        if constexpr (PIPE) {   // probabilities leave as packed (hi, lo) pairs of two positions
-          for (int i = 2 * lane; i < n16; i += 64) {
-            const float2 sv = *reinterpret_cast<const float2*>(row + i);
-            const float e0 = (nm == -INFINITY) ? 0.f : expf(sv.x - nm), e1 = (nm == -INFINITY) ? 0.f : expf(sv.y - nm);
-            const uint32_t hp = pack_bf16(e0, e1);
-            Ph[warp * pw + (i >> 1)] = hp;
-            Pl[warp * pw + (i >> 1)] = pack_bf16(e0 - bf16lo(hp), e1 - bf16hi(hp));
-            sum += e0 + e1;
-          }
-        } else {
-          for (int i = lane; i < n16; i += 32) {
-            const float ex = (nm == -INFINITY) ? 0.f : expf(row[i] - nm);
-            row[i] = ex;
-            sum += ex;
-          }
+        for (int i = lane; i < n16; i += 32) {
+          const float ex = (nm == -INFINITY) ? 0.f : expf(row[i] - nm);
+          row[i] = ex;
+          sum += ex;
         }
 #pragma unroll
         for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
@@ -1201,20 +1132,13 @@ __device__ void attn_phase_mma(const ModelDev& md, int layer, int origin, int ns
         oacc[0] *= r0s; oacc[1] *= r1s; oacc[2] *= r0s; oacc[3] *= r1s;
         for (int kp = 0; kp * 16 < n; ++kp) {
           uint32_t b0 = 0, b1 = 0, b2 = 0, b3 = 0;
-          if constexpr (PIPE) {
-            if (gq < M) {
-              const int w = gq * pw + kp * 8 + tq;
-              b0 = Ph[w]; b1 = Ph[w + 4]; b2 = Pl[w]; b3 = Pl[w + 4];
-            }
-          } else {
-            float2 xa = make_float2(0.f, 0.f), xb = make_float2(0.f, 0.f);
-            if (gq < M) {
-              const float* pr = S + gq * sst + kp * 16 + 2 * tq;
-              xa = *reinterpret_cast<const float2*>(pr);
-              xb = *reinterpret_cast<const float2*>(pr + 8);
-            }
-            split_frag(xa, xb, b0, b1, b2, b3);
+          float2 xa = make_float2(0.f, 0.f), xb = make_float2(0.f, 0.f);
+          if (gq < M) {
+            const float* pr = S + gq * sst + kp * 16 + 2 * tq;
+            xa = *reinterpret_cast<const float2*>(pr);
+            xb = *reinterpret_cast<const float2*>(pr + 8);
           }
+          split_frag(xa, xb, b0, b1, b2, b3);
           // A = V^T: matrices {pos 0-7 x dims 0-7, pos 0-7 x dims 8-15, pos 8-15 x dims 0-7, pos 8-15 x dims 8-15}
           const int r = kp * 16 + (mat >> 1) * 8 + rr;
           const int ch = (warp * 2 + (mat & 1)) ^ (r & 7);
@@ -1225,7 +1149,6 @@ __device__ void attn_phase_mma(const ModelDev& md, int layer, int origin, int ns
         }
       }
       named_sync(1, CONSUMER_THREADS);   // tiles and S are free again
-      if (PIPE) buf ^= 1;
     }
     // oacc[0,1]: dim 16w+gq, queries 2tq, 2tq+1; oacc[2,3]: dim +8
     if (nsplit == 1) {   // the whole context was here: normalise and finish the head
@@ -1233,20 +1156,7 @@ __device__ void attn_phase_mma(const ModelDev& md, int layer, int origin, int ns
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const int q = 2 * tq + (j & 1), c = warp * 16 + gq + (j >> 1) * 8;
-          if (q < M) {
-            const float v = oacc[j] / ctl->rowsum[q];
-            if constexpr (PIPE) {
-              if (o_hi) {
-                const __nv_bfloat16 hv = __float2bfloat16_rn(v);
-                o_hi[(size_t)q * d + h * dh + c] = hv;
-                o_lo[(size_t)q * d + h * dh + c] = __float2bfloat16_rn(v - __bfloat162float(hv));
-              } else {
-                stcg(md.attn + (size_t)q * d + h * dh + c, v);
-              }
-            } else {
-              stcg(md.attn + (size_t)q * d + h * dh + c, v);
-            }
-          }
+          if (q < M) stcg(md.attn + (size_t)q * d + h * dh + c, oacc[j] / ctl->rowsum[q]);
         }
       }
       named_sync(1, CONSUMER_THREADS);
@@ -1273,20 +1183,8 @@ __device__ void attn_phase_mma(const ModelDev& md, int layer, int origin, int ns
       __threadfence();
     }
     named_sync(1, CONSUMER_THREADS);
-    if (ctl->flag) merge_head<M>(md, h, nsplit, reinterpret_cast<float*>(Kt0));
+    if (ctl->flag) merge_head<M>(md, h, nsplit, reinterpret_cast<float*>(Kt));
     named_sync(1, CONSUMER_THREADS);
-    if constexpr (PIPE) {
-      if (ctl->flag && o_hi) {   // the merged rows of this head, once more as bf16 hi + lo
-        for (int i = tid; i < M * dh; i += CONSUMER_THREADS) {
-          const int m = i / dh, c = i - m * dh;
-          const float v = ldcg(md.attn + (size_t)m * d + h * dh + c);
-          const __nv_bfloat16 hv = __float2bfloat16_rn(v);
-          o_hi[(size_t)m * d + h * dh + c] = hv;
-          o_lo[(size_t)m * d + h * dh + c] = __float2bfloat16_rn(v - __bfloat162float(hv));
-        }
-        named_sync(1, CONSUMER_THREADS);
-      }
-    }
   }
 }
 
@@ -1384,8 +1282,10 @@ __device__ void merge_stats(const float* stat_part, int G, int nrows, Ctrl* ctl,
   named_sync(1, CONSUMER_THREADS);
 }
 
+// l / T: the division is exact (and skipped) at T = 1
+__device__ __forceinline__ float div_t(float l, float temperature) { return temperature == 1.0f ? l : __fdiv_rn(l, temperature); }
 __device__ __forceinline__ float prob_of(float logit, float temperature, float rmax, float rsum) {
-  return __fdiv_rn(expf(__fsub_rn(__fdiv_rn(logit, temperature), rmax)), rsum);
+  return __fdiv_rn(expf(__fsub_rn(div_t(logit, temperature), rmax)), rsum);
 }
 
 }  // namespace spd

@@ -4,9 +4,15 @@
 
 namespace spd {
 
+// The words of the device state that a commit updates, read ahead of it.
+struct CommitState { int n_text, pending, block, n_emitted, out_cap; };
+__device__ __forceinline__ CommitState commit_state(const DevState* st) {
+  return CommitState{st->n_text, st->pending, st->block, st->n_emitted, st->out_cap};
+}
+
 // Commit of a step by one thread: accepted count r, next token tok (Sec. 2.1: x_1..x_r and the
 // replacement / bonus token are emitted; the KV length follows the accepted count).
-__device__ __forceinline__ void commit_step(const StepArgs& a, DevState* st, int r, int tok, const int* ids, int pending) {
+__device__ __forceinline__ void commit_step(const StepArgs& a, DevState* st, const CommitState& was, int r, int tok, const int* ids) {
   st->n_acc = r;
   st->next = tok;
   if (a.mode == MODE_ROWS) {           // prefill: the sequence starts here
@@ -15,19 +21,19 @@ __device__ __forceinline__ void commit_step(const StepArgs& a, DevState* st, int
     st->pending = tok;
     st->block = 0;
     st->n_emitted = 0;
-    if (a.out_ids && st->out_cap > 0) { a.out_ids[0] = tok; st->n_emitted = 1; }
+    if (a.out_ids && was.out_cap > 0) { a.out_ids[0] = tok; st->n_emitted = 1; }
   } else {                              // commit x_1..x_r and the next token
-    int ne = st->n_emitted;
+    int ne = was.n_emitted;
     if (a.out_ids) {
       for (int j = 0; j < r; ++j)
-        if (ne < st->out_cap) a.out_ids[ne++] = ids[j];
-      if (ne < st->out_cap) a.out_ids[ne++] = tok;
+        if (ne < was.out_cap) a.out_ids[ne++] = ids[j];
+      if (ne < was.out_cap) a.out_ids[ne++] = tok;
     }
     st->n_emitted = ne;
-    st->n_text += r + 1;
-    st->prev = r >= 1 ? ids[r - 1] : pending;
+    st->n_text = was.n_text + r + 1;
+    st->prev = r >= 1 ? ids[r - 1] : was.pending;
     st->pending = tok;
-    st->block += 1;
+    st->block = was.block + 1;
   }
 }
 
@@ -45,8 +51,8 @@ __device__ void verify_greedy(const StepArgs& a, const ModelDev& md, DevState* s
   int r = gamma;
   for (int j = 0; j < gamma; ++j)
     if (s_arg[j] != ids[j]) { r = j; break; }
-  if (tid == 0) commit_step(a, st, r, s_arg[r], ids, pending);
-  (void)r0;
+  if (tid == 0) commit_step(a, st, commit_state(st), r, s_arg[r], ids);
+  (void)r0; (void)pending;
 }
 
 // Greedy draft step j: x_j = argmax of the row whose statistics sit at index 0.
@@ -307,9 +313,41 @@ __device__ __forceinline__ const float* step_uniforms(const StepArgs& a, const D
   return (a.mode == MODE_VERIFY && a.u_by_block) ? u + a.gamma : u;
 }
 
-// merge_stats by the first 8 warps of a CTA of ROW_THREADS
-__device__ __forceinline__ void merge_stats_rows(const StepArgs& a, int nrows, SampleShared* sh) {
-  if (threadIdx.x < CONSUMER_THREADS) merge_stats(a.md.stat_part, a.fwd_grid, nrows, nullptr, sh->rowmax, sh->rowsum, sh->arg);
+// The row statistics of the forward kernel's slices, merged by the sampling kernels (warp m: row m; the sums
+// in merge_stats' order).  A lane's partials travel together: one memory latency, not five.
+__device__ void merge_stats_rows(const StepArgs& a, int nrows, SampleShared* sh) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, G = a.fwd_grid;
+  if (warp < nrows) {
+    const float4* part = reinterpret_cast<const float4*>(a.md.stat_part) + warp;
+    constexpr int PER = 8;                    // up to 256 slices
+    float4 v[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int c = lane + 32 * i;
+      v[i] = c < G ? __ldcg(part + (size_t)c * MAX_M) : make_float4(-INFINITY, 0.f, -INFINITY, __int_as_float(0x7fffffff));
+    }
+    float mx = -INFINITY, av = -INFINITY, sum = 0.f;
+    int ai = 0x7fffffff;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      mx = fmaxf(mx, v[i].x);
+      const int oi = __float_as_int(v[i].w);
+      if (oi != 0x7fffffff && (ai == 0x7fffffff || v[i].z > av || (v[i].z == av && oi < ai))) { av = v[i].z; ai = oi; }
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      const float ov = __shfl_xor_sync(0xffffffffu, av, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, ai, o);
+      if (oi != 0x7fffffff && (ai == 0x7fffffff || ov > av || (ov == av && oi < ai))) { av = ov; ai = oi; }
+    }
+#pragma unroll
+    for (int i = 0; i < PER; ++i)
+      if (v[i].x != -INFINITY) sum += v[i].y * expf(v[i].x - mx);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) { sh->rowmax[warp] = mx; sh->rowsum[warp] = sum; sh->arg[warp] = ai; }
+  }
   __syncthreads();
 }
 
@@ -320,6 +358,7 @@ __global__ void __launch_bounds__(ROW_THREADS) sample_step_kernel(const __grid_c
   const RowSlice rs = row_slice(C);
   const int V = a.md.V, gamma = a.mode == MODE_VERIFY ? a.gamma : 0, r0 = a.mode == MODE_VERIFY ? 0 : a.sample_r0;
   const float* u = step_uniforms(a, st);
+  const CommitState was = commit_state(st);
   if (threadIdx.x < gamma) {
     const int x = st->d_ids[threadIdx.x];
     s_ids[threadIdx.x] = (unsigned)x < (unsigned)V ? x : 0;   // the forward kernel has flagged it; stay in bounds
@@ -343,7 +382,7 @@ __global__ void __launch_bounds__(ROW_THREADS) sample_step_kernel(const __grid_c
       st->d_ids[a.j] = tok;
       st->t_draft1 = globaltimer();
     } else {
-      commit_step(a, st, r, tok, st->d_ids, st->pending);
+      commit_step(a, st, was, r, tok, st->d_ids);
       if (a.mode == MODE_VERIFY) st->t_verify1 = globaltimer();
     }
   }
@@ -385,6 +424,7 @@ __global__ void __launch_bounds__(ROW_THREADS) sample_rows_kernel(const __grid_c
   const RowSlice rs = row_slice(C);
   const int V = a.md.V;
   const float* u = step_uniforms(a, st);
+  const CommitState was = commit_state(st);
   int r = 0, tok = 0;
   bool mine;
   if (a.mode == MODE_VERIFY) {
@@ -406,7 +446,7 @@ __global__ void __launch_bounds__(ROW_THREADS) sample_rows_kernel(const __grid_c
       st->d_ids[a.j] = tok;
       st->t_draft1 = globaltimer();
     } else {
-      commit_step(a, st, r, tok, st->d_ids, st->pending);
+      commit_step(a, st, was, r, tok, st->d_ids);
       if (a.mode == MODE_VERIFY) st->t_verify1 = globaltimer();
     }
   }

@@ -83,6 +83,7 @@ __global__ void __launch_bounds__(ROW_THREADS) tree_verify_kernel(const __grid_c
   const int V = a.md.V, n = shape.n, tid = threadIdx.x;
   const RowSlice rs{0, 1};      // one CTA: the walk is a chain of decisions
   const float* u = step_uniforms(a, st);
+  const CommitState was = commit_state(st);
   if (tid < n) {
     const int x = st->d_ids[tid];
     s_ids[tid] = (unsigned)x < (unsigned)V ? x : 0;   // the forward kernel has flagged it
@@ -138,7 +139,7 @@ __global__ void __launch_bounds__(ROW_THREADS) tree_verify_kernel(const __grid_c
   __syncthreads();
   if (tid == 0) {
     for (int j = 0; j < plen; ++j) st->path[j] = s_path[j];
-    commit_step(a, st, plen, tok, s_path_ids, st->pending);
+    commit_step(a, st, was, plen, tok, s_path_ids);
     st->t_verify1 = globaltimer();
   }
 }
