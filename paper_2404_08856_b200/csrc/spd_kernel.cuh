@@ -47,7 +47,8 @@ __device__ void verify_greedy(const StepArgs& a, const ModelDev& md, DevState* s
                               int gamma, const int* ids /*gamma draft ids*/, int pending) {
   const int tid = threadIdx.x;
   __shared__ int s_arg[MAX_M];
-  merge_stats(md.stat_part, G, gamma + 1, ctl, ctl->rowmax, ctl->rowsum, s_arg);
+  merge_stats(md.stat_part, G, gamma + 1, ctl->rowmax, ctl->rowsum, s_arg);
+  named_sync(1, CONSUMER_THREADS);
   int r = gamma;
   for (int j = 0; j < gamma; ++j)
     if (s_arg[j] != ids[j]) { r = j; break; }
@@ -59,7 +60,8 @@ __device__ void verify_greedy(const StepArgs& a, const ModelDev& md, DevState* s
 template <int M>
 __device__ void draft_greedy(const StepArgs& a, const ModelDev& md, DevState* st, Ctrl* ctl, int G) {
   __shared__ int s_arg[MAX_M];
-  merge_stats(md.stat_part, G, 1, ctl, ctl->rowmax, ctl->rowsum, s_arg);
+  merge_stats(md.stat_part, G, 1, ctl->rowmax, ctl->rowsum, s_arg);
+  named_sync(1, CONSUMER_THREADS);
   if (threadIdx.x == 0) st->d_ids[a.j] = s_arg[0];
 }
 
@@ -246,7 +248,7 @@ __global__ void __launch_bounds__(ENGINE_THREADS, 1) forward_kernel(const __grid
       }
       if (want_head) {
         // row statistics over vocabulary slices, then CTA 0 applies the sampling rule
-        stats_phase<M>(a.logits, md.V, a.stat_r0, a.stat_n, a.temperature, cta, G, md.stat_part, ctl);
+        stats_phase<M>(a.logits, md.V, a.stat_r0, a.stat_n, a.temperature, cta, G, md.stat_part);
         stamp(3); sync_grid(); stamp(4);
         if (cta == 0 && a.greedy && !a.tree) {
           if (a.mode == MODE_VERIFY) verify_greedy<M>(a, md, st, ctl, G, 0, a.gamma, ctl->tok + 1, pending);
@@ -313,41 +315,8 @@ __device__ __forceinline__ const float* step_uniforms(const StepArgs& a, const D
   return (a.mode == MODE_VERIFY && a.u_by_block) ? u + a.gamma : u;
 }
 
-// The row statistics of the forward kernel's slices, merged by the sampling kernels (warp m: row m; the sums
-// in merge_stats' order).  A lane's partials travel together: one memory latency, not five.
-__device__ void merge_stats_rows(const StepArgs& a, int nrows, SampleShared* sh) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, G = a.fwd_grid;
-  if (warp < nrows) {
-    const float4* part = reinterpret_cast<const float4*>(a.md.stat_part) + warp;
-    constexpr int PER = 8;                    // up to 256 slices
-    float4 v[PER];
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-      const int c = lane + 32 * i;
-      v[i] = c < G ? __ldcg(part + (size_t)c * MAX_M) : make_float4(-INFINITY, 0.f, -INFINITY, __int_as_float(0x7fffffff));
-    }
-    float mx = -INFINITY, av = -INFINITY, sum = 0.f;
-    int ai = 0x7fffffff;
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-      mx = fmaxf(mx, v[i].x);
-      const int oi = __float_as_int(v[i].w);
-      if (oi != 0x7fffffff && (ai == 0x7fffffff || v[i].z > av || (v[i].z == av && oi < ai))) { av = v[i].z; ai = oi; }
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      const float ov = __shfl_xor_sync(0xffffffffu, av, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, ai, o);
-      if (oi != 0x7fffffff && (ai == 0x7fffffff || ov > av || (ov == av && oi < ai))) { av = ov; ai = oi; }
-    }
-#pragma unroll
-    for (int i = 0; i < PER; ++i)
-      if (v[i].x != -INFINITY) sum += v[i].y * expf(v[i].x - mx);
-#pragma unroll
-    for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (lane == 0) { sh->rowmax[warp] = mx; sh->rowsum[warp] = sum; sh->arg[warp] = ai; }
-  }
+__device__ __forceinline__ void merge_stats_rows(const StepArgs& a, int nrows, SampleShared* sh) {
+  merge_stats(a.md.stat_part, a.fwd_grid, nrows, sh->rowmax, sh->rowsum, sh->arg);
   __syncthreads();
 }
 
@@ -406,7 +375,7 @@ __global__ void __launch_bounds__(PROB_THREADS) prob_rows_kernel(const __grid_co
   const int cta = blockIdx.x, G = gridDim.x, V = a.md.V;
   const int nrows = a.stat_n, r0 = a.stat_r0;
   // the statistics of row r0 + r sit at index r
-  merge_stats(a.md.stat_part, a.fwd_grid, nrows, nullptr, sh.rowmax, sh.rowsum, sh.arg);
+  merge_stats_rows(a, nrows, &sh);
   const int VS = (V + G - 1) / G;
   const int k0 = cta * VS, k1 = min(V, k0 + VS);
   for (int r = 0; r < nrows; ++r) {

@@ -11,13 +11,6 @@
 
 namespace spd {
 
-// scratch of the forward kernel's own row statistics
-struct SampleScratch {
-  float amax[8];
-  int aidx[8];
-  float fval[8];
-};
-
 __device__ __forceinline__ unsigned long long to_fixed(float w) {
   return static_cast<unsigned long long>(__fmul_rn(w, 4294967296.0f));  // cvt.rzi, exact scale
 }
