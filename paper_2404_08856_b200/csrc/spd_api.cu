@@ -50,8 +50,7 @@ struct spd_ctx {
   int device = 0, n_sm = 0, smem_optin = 0;
   ModelHost target, draft;
   DevState* st = nullptr;
-  unsigned* bars = nullptr;     // pool of grid-barrier counters
-  int bar_next = 0;
+  unsigned* bars = nullptr;     // grid barrier of the forward launches, then (BAR_WORDS on) the self-test's
   float* ubuf = nullptr;        // [16] uniforms of direct calls: [0..7] draft, [8..15] verify
   float* qbuf = nullptr;        // [gamma_max][V] draft distributions
   float* prow = nullptr;        // [MAX_M][V] probability rows of the step being sampled (top-k / top-p only)
@@ -103,7 +102,7 @@ struct spd_ctx {
 
 namespace {
 
-constexpr int BAR_POOL = 64;
+constexpr int BAR_WORDS = 64;     // counter and base, 128 bytes apart
 
 spd_status fail(spd_ctx* c, spd_status s, const std::string& msg) {
   if (c) c->err = msg;
@@ -444,8 +443,6 @@ spd_status launch_cfg(spd_ctx* ctx, KernelFn fn, int M, int n_sm, int smem_optin
   return SPD_OK;
 }
 
-unsigned* next_bar(spd_ctx* ctx);
-
 // One cluster of `cs` CTAs with this kernel's shared memory must be able to run.
 bool cluster_fits(KernelFn fn, int cs, size_t smem) {
   if (cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
@@ -515,7 +512,6 @@ spd_status launch_forward(spd_ctx* ctx, int M, int dtype, StepArgs a, cudaStream
     cfg.attrs = at; cfg.numAttrs = 1;
     CU(cudaLaunchKernelExC(&cfg, (const void*)fn, params));
   } else {
-    CU(cudaMemsetAsync(bar, 0, sizeof(unsigned), stream));
     CU(cudaLaunchCooperativeKernel((const void*)fn, dim3(grid), dim3(ENGINE_THREADS), params, lc.smem, stream));
   }
   // sampling (not greedy): the forward kernel has left logits and per-slice row statistics; a small
@@ -539,13 +535,7 @@ spd_status launch_forward(spd_ctx* ctx, int M, int dtype, StepArgs a, cudaStream
 }
 
 spd_status launch_model(spd_ctx* ctx, ModelHost& mh, int M, StepArgs a, cudaStream_t stream) {
-  return launch_forward(ctx, M, mh.cfg.dtype, a, stream, mh.grid, mh.cluster, ctx->smem_optin, next_bar(ctx), ctx->n_sm);
-}
-
-unsigned* next_bar(spd_ctx* ctx) {
-  unsigned* b = ctx->bars + 32 * (ctx->bar_next % BAR_POOL);  // 128 B apart
-  ctx->bar_next++;
-  return b;
+  return launch_forward(ctx, M, mh.cfg.dtype, a, stream, mh.grid, mh.cluster, ctx->smem_optin, ctx->bars, ctx->n_sm);
 }
 
 spd_status check_dev_err(spd_ctx* ctx, int e) {
@@ -560,22 +550,25 @@ spd_status sync_state(spd_ctx* ctx, cudaStream_t stream = nullptr, bool use_give
   CU(cudaStreamSynchronize(cs));
   ctx->len_ub = ctx->st_host->n_text;
   const int e = ctx->st_host->err;
-  if (e != DEV_OK) {
+  if (e != DEV_OK) {   // (a barrier that gave up leaves its count anywhere)
     cudaMemsetAsync(&ctx->st->err, 0, sizeof(int), ctx->stream);
+    cudaMemsetAsync(ctx->bars, 0, BAR_WORDS * sizeof(unsigned), ctx->stream);
     return check_dev_err(ctx, e);
   }
   return SPD_OK;
 }
 
-spd_status copy_out(spd_ctx* ctx, void* dst, const void* src_dev, size_t bytes, bool* need_sync) {
+// Results that live in the device state.  Device destinations are copied on the stream at once; for host
+// destinations the caller reads the whole state back with one pinned copy (sync_state) and hands
+// them out with put_result: a copy per word into pageable memory would block for each.
+spd_status copy_result(spd_ctx* ctx, void* dst, const void* src_dev, size_t bytes, bool* to_host) {
   if (!dst) return SPD_OK;
-  if (is_device_ptr(dst)) {
-    CU(cudaMemcpyAsync(dst, src_dev, bytes, cudaMemcpyDeviceToDevice, ctx->stream));
-  } else {
-    CU(cudaMemcpyAsync(dst, src_dev, bytes, cudaMemcpyDeviceToHost, ctx->stream));
-    *need_sync = true;
-  }
+  if (is_device_ptr(dst)) CU(cudaMemcpyAsync(dst, src_dev, bytes, cudaMemcpyDeviceToDevice, ctx->stream));
+  else *to_host = true;
   return SPD_OK;
+}
+void put_result(void* dst, const void* src_host, size_t bytes) {
+  if (dst && !is_device_ptr(dst)) memcpy(dst, src_host, bytes);
 }
 
 // Row tables of the two plain launches (spd_engine.cuh, RowGeom).  Verify: the chain
@@ -766,6 +759,12 @@ spd_status ug_gemm(spd_ctx* ctx, const __nv_bfloat16* x_hi, const __nv_bfloat16*
   return ug_launch<1, UG_SWIGLU>(ctx, mw, mh, ml, a);
 }
 
+__global__ void set_sequence_kernel(DevState* st, int n_text, int pending, int prev) {
+  st->n_text = n_text;
+  st->pending = pending;
+  st->prev = prev;
+}
+
 // Embedding rows of n token ids.  An id outside [0, V) (possible when the ids live in device
 // memory, which the host cannot inspect) is read as token 0 and recorded in *err.
 __global__ void gather_rows_kernel(const int* ids, const float* table, float* out, int n, int d, int V, int* err) {
@@ -873,7 +872,7 @@ spd_status alloc_ctx_buffers(spd_ctx* ctx) {
   const int dmax = cfg->target.d_model > cfg->draft.d_model ? cfg->target.d_model : cfg->draft.d_model;
   spd_status s;
   if ((s = dalloc(ctx, &ctx->st, 1))) return s;
-  if ((s = dalloc(ctx, &ctx->bars, (size_t)32 * BAR_POOL))) return s;
+  if ((s = dalloc(ctx, &ctx->bars, (size_t)2 * BAR_WORDS))) return s;
   if ((s = dalloc(ctx, &ctx->ubuf, 16))) return s;
   if ((s = dalloc(ctx, &ctx->qbuf, (size_t)MAX_M * V))) return s;   // chain: gamma rows; tree: one per block row
   ctx->truncate = !cfg->greedy && ((cfg->top_k >= 1 && cfg->top_k < V) || (cfg->top_p > 0.f && cfg->top_p < 1.f));
@@ -1207,6 +1206,7 @@ spd_status spd_image_adapter(spd_ctx* ctx, const float* feats, int m, int d_in, 
   CU(cudaStreamSynchronize(ctx->stream));
   if (e != DEV_OK) {
     cudaMemsetAsync(&ctx->st->err, 0, sizeof(int), ctx->stream);
+    cudaMemsetAsync(ctx->bars, 0, BAR_WORDS * sizeof(unsigned), ctx->stream);
     return check_dev_err(ctx, e);
   }
   return SPD_OK;
@@ -1233,13 +1233,11 @@ spd_status spd_draft(spd_ctx* ctx, int gamma, const float* uniforms, int32_t* dr
     geom_draft_step(a, j);
     a.uniforms = ctx->ubuf;
     a.q_out = ctx->qbuf;
-    a.logits = dm.logits;
+    // the launch's two logits rows go to rows 6-j and 7-j of the buffer: the step's own row (the second)
+    // stays for spd_get_draft_logits, its first row is overwritten by the next step's second
+    a.logits = dm.logits + (size_t)(MAX_M - 2 - j) * dm.cfg.vocab;
     spd_status s = launch_model(ctx, dm, 2, a, ctx->stream);
     if (s) return s;
-    // keep this step's logits row (row 1) for spd_get_draft_logits: rows 2.. of the buffer
-    if (j + 2 < MAX_M)
-      CU(cudaMemcpyAsync(dm.logits + (size_t)(j + 2) * dm.cfg.vocab, dm.logits + (size_t)dm.cfg.vocab,
-                         dm.cfg.vocab * sizeof(float), cudaMemcpyDeviceToDevice, ctx->stream));
   }
   ctx->drafted_gamma = gamma;
   ctx->last_draft_rows = gamma < MAX_M - 2 ? gamma : MAX_M - 2;
@@ -1247,8 +1245,12 @@ spd_status spd_draft(spd_ctx* ctx, int gamma, const float* uniforms, int32_t* dr
   spd_status s;
   if (draft_probs && !ctx->cfg.greedy)
     CU(cudaMemcpyAsync(draft_probs, ctx->qbuf, (size_t)gamma * dm.cfg.vocab * sizeof(float), cudaMemcpyDeviceToDevice, ctx->stream));
-  if ((s = copy_out(ctx, draft_ids, ctx->st->d_ids, gamma * sizeof(int32_t), &need_sync))) return s;
-  if (need_sync) CU(cudaStreamSynchronize(ctx->stream));
+  if ((s = copy_result(ctx, draft_ids, ctx->st->d_ids, gamma * sizeof(int32_t), &need_sync))) return s;
+  if (need_sync) {
+    CU(cudaMemcpyAsync(ctx->st_host->d_ids, ctx->st->d_ids, sizeof(ctx->st->d_ids), cudaMemcpyDeviceToHost, ctx->stream));
+    CU(cudaStreamSynchronize(ctx->stream));
+    put_result(draft_ids, ctx->st_host->d_ids, gamma * sizeof(int32_t));
+  }
   return SPD_OK;
 }
 
@@ -1289,10 +1291,13 @@ spd_status spd_verify(spd_ctx* ctx, int gamma, const int32_t* draft_ids, const f
   ctx->len_ub += gamma + 1;
   ctx->last_verify_rows = gamma + 1;
   bool need_sync = false;
-  if ((s = copy_out(ctx, n_accepted, &ctx->st->n_acc, sizeof(int32_t), &need_sync))) return s;
-  if ((s = copy_out(ctx, next_token, &ctx->st->next, sizeof(int32_t), &need_sync))) return s;
-  if (need_sync) return sync_state(ctx);
-  return SPD_OK;
+  if ((s = copy_result(ctx, n_accepted, &ctx->st->n_acc, sizeof(int32_t), &need_sync))) return s;
+  if ((s = copy_result(ctx, next_token, &ctx->st->next, sizeof(int32_t), &need_sync))) return s;
+  if (!need_sync) return SPD_OK;
+  s = sync_state(ctx);
+  put_result(n_accepted, &ctx->st_host->n_acc, sizeof(int32_t));
+  put_result(next_token, &ctx->st_host->next, sizeof(int32_t));
+  return s;
 }
 
 // ---- tree blocks
@@ -1397,9 +1402,13 @@ spd_status spd_draft_tree(spd_ctx* ctx, int depth, const int32_t* branching, con
   bool need_sync = false;
   if (draft_probs && !ctx->cfg.greedy)
     CU(cudaMemcpyAsync(draft_probs, ctx->qbuf, (size_t)(n + 1) * dm.cfg.vocab * sizeof(float), cudaMemcpyDeviceToDevice, ctx->stream));
-  if ((s = copy_out(ctx, node_ids, ctx->st->d_ids, n * sizeof(int32_t), &need_sync))) return s;
+  if ((s = copy_result(ctx, node_ids, ctx->st->d_ids, n * sizeof(int32_t), &need_sync))) return s;
   if (parent_out) memcpy(parent_out, parent, (n + 1) * sizeof(int32_t));
-  if (need_sync) CU(cudaStreamSynchronize(ctx->stream));
+  if (need_sync) {
+    CU(cudaMemcpyAsync(ctx->st_host->d_ids, ctx->st->d_ids, sizeof(ctx->st->d_ids), cudaMemcpyDeviceToHost, ctx->stream));
+    CU(cudaStreamSynchronize(ctx->stream));
+    put_result(node_ids, ctx->st_host->d_ids, n * sizeof(int32_t));
+  }
   return SPD_OK;
 }
 
@@ -1463,11 +1472,15 @@ spd_status spd_verify_tree(spd_ctx* ctx, int n_nodes, const int32_t* parent, con
   ctx->len_ub += sh.depth_max + 1;
   ctx->last_verify_rows = n + 1;
   bool need_sync = false;
-  if ((s = copy_out(ctx, n_accepted, &ctx->st->n_acc, sizeof(int32_t), &need_sync))) return s;
-  if ((s = copy_out(ctx, next_token, &ctx->st->next, sizeof(int32_t), &need_sync))) return s;
-  if ((s = copy_out(ctx, path, ctx->st->path, sh.depth_max * sizeof(int32_t), &need_sync))) return s;
-  if (need_sync) return sync_state(ctx);
-  return SPD_OK;
+  if ((s = copy_result(ctx, n_accepted, &ctx->st->n_acc, sizeof(int32_t), &need_sync))) return s;
+  if ((s = copy_result(ctx, next_token, &ctx->st->next, sizeof(int32_t), &need_sync))) return s;
+  if ((s = copy_result(ctx, path, ctx->st->path, sh.depth_max * sizeof(int32_t), &need_sync))) return s;
+  if (!need_sync) return SPD_OK;
+  s = sync_state(ctx);
+  put_result(n_accepted, &ctx->st_host->n_acc, sizeof(int32_t));
+  put_result(next_token, &ctx->st_host->next, sizeof(int32_t));
+  put_result(path, ctx->st_host->path, sh.depth_max * sizeof(int32_t));
+  return s;
 }
 
 // ---- several sequences in one pass over the weights
@@ -1480,7 +1493,10 @@ struct spd_batch {
   int B = 0;
   BatchSeq* seqs_dev = nullptr;
   ModelDev *mds_t = nullptr, *mds_d = nullptr;
-  int *rowslot = nullptr, *origins = nullptr, *out_acc = nullptr, *out_next = nullptr;
+  int *rowslot = nullptr, *origins = nullptr;
+  int *out_dev = nullptr, *out_host = nullptr;   // [B] accepted, [B] next, [B][MAX_M] draft ids; the host copy is pinned
+  std::vector<BatchSeq> h_seqs;                  // the descriptors as uploaded last
+  std::vector<ModelDev> h_t, h_d;
   RowStats* stats = nullptr;    // (max, sum exp) of the rows of a verify step
   float *part_o = nullptr, *part_ml = nullptr;   // attention partials of the KV splits
   unsigned* attn_cnt = nullptr;
@@ -1605,6 +1621,16 @@ spd_status batch_room(spd_batch* bt, int rows, bool draft) {
   return SPD_OK;
 }
 
+// Uploads descriptors that differ from what the device has.
+template <class T>
+spd_status upload_changed(spd_ctx* ctx, T* dev, std::vector<T>& have, const std::vector<T>& now) {
+  if (have.size() == now.size() && !memcmp(have.data(), now.data(), now.size() * sizeof(T))) return SPD_OK;
+  have = now;
+  CU(cudaMemcpyAsync(dev, have.data(), have.size() * sizeof(T), cudaMemcpyHostToDevice, ctx->stream));
+  CU(cudaStreamSynchronize(ctx->stream));
+  return SPD_OK;
+}
+
 // Runs `enqueue` (which issues its launches on ctx->stream) either directly or, from its second use
 // on, as a replay of the graph captured from it.  The first use runs eagerly so that one-time set-up
 // (scratch growth, kernel attributes) happens outside any capture.
@@ -1653,6 +1679,7 @@ void spd_batch_destroy(spd_batch* bt) {
     if (g.exec) cudaGraphExecDestroy(g.exec);
   if (bt->cap_stream) cudaStreamDestroy(bt->cap_stream);
   for (void* p : bt->allocs) cudaFree(p);
+  if (bt->out_host) cudaFreeHost(bt->out_host);
   delete bt;
 }
 
@@ -1688,8 +1715,9 @@ spd_status spd_batch_create(spd_ctx* const* seqs, int B, spd_batch** out) {
   if (!s) s = balloc(bt, &bt->mds_d, (size_t)B);
   if (!s) s = balloc(bt, &bt->rowslot, (size_t)BATCH_ROWS_MAX);
   if (!s) s = balloc(bt, &bt->origins, (size_t)B);
-  if (!s) s = balloc(bt, &bt->out_acc, (size_t)B);
-  if (!s) s = balloc(bt, &bt->out_next, (size_t)B);
+  if (!s) s = balloc(bt, &bt->out_dev, (size_t)B * (2 + MAX_M));
+  if (!s && cudaMallocHost(&bt->out_host, (size_t)B * (2 + MAX_M) * sizeof(int)) != cudaSuccess)
+    s = fail(ctx, SPD_ENOMEM, "pinned allocation failed");
   if (!s) s = balloc(bt, &bt->X, (size_t)BATCH_ROWS_MAX * dmax);
   if (!s) s = balloc(bt, &bt->logits, (size_t)BATCH_ROWS_MAX * V);
   if (!s) s = balloc(bt, &bt->stats, (size_t)BATCH_ROWS_MAX);
@@ -1715,7 +1743,8 @@ spd_status spd_batch_create(spd_ctx* const* seqs, int B, spd_batch** out) {
   return SPD_OK;
 }
 
-// (re)reads each sequence's descriptors: a prefill changes the rows in front of the text
+// (re)reads each sequence's descriptors -- a prefill changes the rows in front of the text -- and uploads
+// them where they differ from what the device has
 static spd_status batch_refresh(spd_batch* bt) {
   spd_ctx* ctx = bt->lead;
   std::vector<BatchSeq> hs(bt->B);
@@ -1724,14 +1753,13 @@ static spd_status batch_refresh(spd_batch* bt) {
     spd_ctx* c = bt->seqs[b];
     if (!c->prefilled) return fail(ctx, SPD_ESTATE, "a sequence of the batch has not been prefilled");
     hs[b] = BatchSeq{c->st, c->target.pos_base, c->draft.pos_base};
-    ht[b] = c->target.md;
-    hd[b] = c->draft.md;
+    memcpy(&ht[b], &c->target.md, sizeof(ModelDev));   // (with its padding: compared as bytes)
+    memcpy(&hd[b], &c->draft.md, sizeof(ModelDev));
   }
-  CU(cudaMemcpyAsync(bt->seqs_dev, hs.data(), hs.size() * sizeof(BatchSeq), cudaMemcpyHostToDevice, ctx->stream));
-  CU(cudaMemcpyAsync(bt->mds_t, ht.data(), ht.size() * sizeof(ModelDev), cudaMemcpyHostToDevice, ctx->stream));
-  CU(cudaMemcpyAsync(bt->mds_d, hd.data(), hd.size() * sizeof(ModelDev), cudaMemcpyHostToDevice, ctx->stream));
-  CU(cudaStreamSynchronize(ctx->stream));   // the host vectors go out of scope
-  return SPD_OK;
+  spd_status s;
+  if ((s = upload_changed(ctx, bt->seqs_dev, bt->h_seqs, hs))) return s;
+  if ((s = upload_changed(ctx, bt->mds_t, bt->h_t, ht))) return s;
+  return upload_changed(ctx, bt->mds_d, bt->h_d, hd);
 }
 
 spd_status spd_batch_draft(spd_batch* bt, int gamma, const float* uniforms, int32_t* draft_ids) {
@@ -1752,7 +1780,7 @@ spd_status spd_batch_draft(spd_batch* bt, int gamma, const float* uniforms, int3
       if (ctx->truncate && (r = batch_probs(bt, B, 1, 2))) return r;
       const int C = row_ctas(ctx->n_sm, B, V);
       CU(launch_rows(batch_draft_sample_kernel, B, C, ROW_THREADS, ctx->stream, true, bt->seqs_dev, C, bt->logits,
-                     ctx->truncate ? bt->probs : nullptr, V, gamma, j, ctx->cfg.greedy, ctx->cfg.temperature, bt->u_draft, bt->q_all));
+                     ctx->truncate ? bt->probs : nullptr, V, gamma, j, ctx->cfg.greedy, ctx->cfg.temperature, bt->u_draft, bt->q_all, bt->out_dev + 2 * B));
       return SPD_OK;
     };
     if ((s = run_step_graph(bt, bt->g_draft[gamma][j], step))) return s;
@@ -1760,11 +1788,15 @@ spd_status spd_batch_draft(spd_batch* bt, int gamma, const float* uniforms, int3
   bt->last_rows = 2 * B;
   bt->drafted_gamma = gamma;
   for (spd_ctx* c : bt->seqs) { c->drafted_gamma = -1; c->tree_drafted = false; }
-  if (draft_ids) {
-    const bool host = !is_device_ptr(draft_ids);
-    for (int b = 0; b < B; ++b)
-      CU(cudaMemcpyAsync(draft_ids + (size_t)b * gamma, bt->seqs[b]->st->d_ids, gamma * sizeof(int32_t), cudaMemcpyDefault, ctx->stream));
-    if (host) CU(cudaStreamSynchronize(ctx->stream));
+  if (draft_ids) {      // the ids of all sequences sit together, [B][gamma]
+    const size_t bytes = (size_t)B * gamma * sizeof(int32_t);
+    if (is_device_ptr(draft_ids)) {
+      CU(cudaMemcpyAsync(draft_ids, bt->out_dev + 2 * B, bytes, cudaMemcpyDeviceToDevice, ctx->stream));
+    } else {
+      CU(cudaMemcpyAsync(bt->out_host + 2 * B, bt->out_dev + 2 * B, bytes, cudaMemcpyDeviceToHost, ctx->stream));
+      CU(cudaStreamSynchronize(ctx->stream));
+      memcpy(draft_ids, bt->out_host + 2 * B, bytes);
+    }
   }
   return SPD_OK;
 }
@@ -1787,7 +1819,7 @@ spd_status spd_batch_verify(spd_batch* bt, int gamma, const float* uniforms, int
     const int C = row_ctas(ctx->n_sm, B, V);
     CU(launch_rows(batch_verify_kernel, B, C, ROW_THREADS, ctx->stream, true, bt->seqs_dev, C, bt->logits, bt->stats,
                    ctx->truncate ? bt->probs : nullptr, bt->q_all, ctx->cfg.greedy ? nullptr : bt->u_verify, gamma, V,
-                   ctx->cfg.greedy, ctx->cfg.temperature, bt->out_acc, bt->out_next));
+                   ctx->cfg.greedy, ctx->cfg.temperature, bt->out_dev, bt->out_dev + B));
     return SPD_OK;
   };
   if ((s = run_step_graph(bt, bt->g_verify[gamma], step))) return s;
@@ -1795,10 +1827,14 @@ spd_status spd_batch_verify(spd_batch* bt, int gamma, const float* uniforms, int
   bt->drafted_gamma = -1;
   for (spd_ctx* c : bt->seqs) { c->len_ub += M; c->drafted_gamma = -1; c->last_verify_rows = 0; }
   bool need_sync = false;
-  if ((s = copy_out(ctx, n_accepted, bt->out_acc, B * sizeof(int32_t), &need_sync))) return s;
-  if ((s = copy_out(ctx, next_token, bt->out_next, B * sizeof(int32_t), &need_sync))) return s;
-  if (need_sync) return sync_state(ctx);   // also reports a device-side error (bad id, a wait that ran out)
-  return SPD_OK;
+  if ((s = copy_result(ctx, n_accepted, bt->out_dev, B * sizeof(int32_t), &need_sync))) return s;
+  if ((s = copy_result(ctx, next_token, bt->out_dev + B, B * sizeof(int32_t), &need_sync))) return s;
+  if (!need_sync) return SPD_OK;
+  CU(cudaMemcpyAsync(bt->out_host, bt->out_dev, (size_t)2 * B * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  s = sync_state(ctx);   // also reports a device-side error (bad id, a wait that ran out)
+  put_result(n_accepted, bt->out_host, B * sizeof(int32_t));
+  put_result(next_token, bt->out_host + B, B * sizeof(int32_t));
+  return s;
 }
 
 spd_status spd_batch_get_logits(spd_batch* bt, float* logits, int rows) {
@@ -1941,7 +1977,9 @@ spd_status spd_get_draft_logits(spd_ctx* ctx, float* logits, int rows) {
   if (!ctx || !logits) return SPD_EINVAL;
   if (rows < 1 || rows > ctx->last_draft_rows) return fail(ctx, SPD_EINVAL, "rows exceed the last draft call");
   const int V = ctx->cfg.draft.vocab;
-  CU(cudaMemcpyAsync(logits, ctx->draft.logits + (size_t)2 * V, (size_t)rows * V * sizeof(float), cudaMemcpyDefault, ctx->stream));
+  for (int j = 0; j < rows; ++j)   // (spd_draft leaves step j's row at 7 - j)
+    CU(cudaMemcpyAsync(logits + (size_t)j * V, ctx->draft.logits + (size_t)(MAX_M - 1 - j) * V, V * sizeof(float), cudaMemcpyDefault,
+                       ctx->stream));
   CU(cudaStreamSynchronize(ctx->stream));
   return SPD_OK;
 }
@@ -1972,9 +2010,9 @@ spd_status spd_rollback(spd_ctx* ctx, int n_text, int32_t prev_token, int32_t pe
   if (n_text < 1 || ctx->m_image + n_text + 1 > ctx->cfg.max_seq || prev_token < 0 || prev_token >= V ||
       pending_token < 0 || pending_token >= V)
     return fail(ctx, SPD_EINVAL, "bad rollback arguments");
-  int v[3] = {n_text, pending_token, prev_token};
-  CU(cudaMemcpyAsync(&ctx->st->n_text, v, sizeof(v), cudaMemcpyHostToDevice, ctx->stream));
-  CU(cudaStreamSynchronize(ctx->stream));
+  // (three words by value: a copy from the host would have to wait for the stream)
+  set_sequence_kernel<<<1, 1, 0, ctx->stream>>>(ctx->st, n_text, pending_token, prev_token);
+  CU(cudaGetLastError());
   ctx->len_ub = n_text;
   ctx->drafted_gamma = -1;
   return SPD_OK;
@@ -2025,7 +2063,7 @@ spd_status spd_truncate_probs(const float* probs, float* out, int rows, int V, i
   return cudaGetLastError() == cudaSuccess ? SPD_OK : SPD_ECUDA;
 }
 
-// Scratch of the two stand-alone GEMM entry points, per device: a grid-barrier word, a status
+// Scratch of the two stand-alone GEMM entry points, per device: a status
 // block (DevState: only its error word is used) and, for spd_skinny_gemm, the tile-packed copy of w.
 struct GemmScratch {
   bool ready = false;
@@ -2122,8 +2160,7 @@ spd_status spd_skinny_gemm_noalloc(const float* x, const void* w, int dtype, int
   }
   spd_ctx* ctx = nullptr;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
-  // the array keeps whatever the last call left: the barrier word and the status block must
-  // start at zero (launch_forward clears the barrier word, the status block is cleared here)
+  // the array keeps whatever the last call left: the status block must start at zero
   if (cudaMemsetAsync(g.st, 0, 256, cs) != cudaSuccess) return SPD_ECUDA;
   spd_status s = pack_tiles(ctx, g.packed, w, N, K, esz, g.n_sm, cs);
   if (s) return s;
@@ -2137,7 +2174,7 @@ spd_status spd_skinny_gemm_noalloc(const float* x, const void* w, int dtype, int
 spd_status spd_wait_selftest(spd_ctx* ctx, int which, unsigned polls) {
   if (!ctx) return SPD_EINVAL;
   if ((which != 0 && which != 1) || polls < 1 || polls > (1u << 20)) return fail(ctx, SPD_EINVAL, "bad selftest arguments");
-  unsigned* bar = next_bar(ctx);
+  unsigned* bar = ctx->bars + BAR_WORDS;
   CU(cudaMemsetAsync(bar, 0, sizeof(unsigned), ctx->stream));
   wait_selftest_kernel<<<ctx->n_sm, CONSUMER_THREADS, 0, ctx->stream>>>(ctx->st, bar, which, polls);
   CU(cudaGetLastError());

@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(ROW_THREADS) batch_softmax_kernel(const float*
 // sequence's draft distributions [B][gamma][V].  probs: the truncated rows [B][V], or NULL.
 __global__ void __launch_bounds__(ROW_THREADS) batch_draft_sample_kernel(const BatchSeq* seqs, int C,
                                                                          const float* logits, const float* probs, int V, int gamma, int j, int greedy,
-                                                                         float temperature, const float* u, float* q_all) {
+                                                                         float temperature, const float* u, float* q_all, int* ids_out) {
   __shared__ RowScratch sc;
   __shared__ StatScratch ss;
   const RowSlice rs = row_slice(C);
@@ -375,7 +375,10 @@ __global__ void __launch_bounds__(ROW_THREADS) batch_draft_sample_kernel(const B
     const unsigned long long Z = row_mass(wf, [&](int k, float w) { stcg(q + k, w); }, V, rs, &sc);
     mine = row_pick(wf, V, Z, u[(size_t)b * gamma + j], rs, &sc, tok);
   }
-  if (mine && threadIdx.x == 0) seqs[b].st->d_ids[j] = tok;
+  if (mine && threadIdx.x == 0) {
+    seqs[b].st->d_ids[j] = tok;
+    ids_out[b * gamma + j] = tok;      // all sequences' ids together for the caller
+  }
 }
 
 // The rejection rule and the commit, C CTAs per sequence (Sec. 2.1): the target's rows are logits

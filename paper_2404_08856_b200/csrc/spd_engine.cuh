@@ -50,6 +50,8 @@ __host__ __device__ constexpr int x_bytes(int M) {
   return M * (KC_MAX + X_PAD) * 4 > 65536 ? M * (KC_MAX + X_PAD) * 4 : 65536;
 }
 
+constexpr int BAR_BASE = 32;          // 128 bytes away from the counter
+
 enum : int { MODE_VERIFY = 0, MODE_DRAFT = 1, MODE_ROWS = 2, MODE_GEMM = 3 };
 enum : int { PRO_PLAIN = 0, PRO_NORM = 1 };
 enum : int { EPI_STORE = 0, EPI_RESID = 1, EPI_SWIGLU = 2, EPI_QKV = 3 };
@@ -120,7 +122,7 @@ struct StepArgs {
   int stat_r0, stat_n;    // rows of `logits` whose softmax statistics the kernel leaves for the sampling kernels
   int tree;               // 1: a tree block -- the rule runs in the tree kernels, never inside this kernel
   DevState* st;
-  unsigned* bar;          // grid-barrier counter, zero at launch
+  unsigned* bar;          // grid barrier: [0] arrivals, [BAR_BASE] their number before this launch
   int mode, gamma, j, pos_base, nstage, greedy;
   int cluster_ctas;       // > 0: the grid is ONE thread-block cluster of that many CTAs (small models)
   int fwd_grid;           // CTAs of the forward kernel that left the row statistics (set at launch)
@@ -693,6 +695,9 @@ __device__ void consume_gemm(const Gemm& g, const EpiArgs& e, const XSrc& src, c
 }
 
 // ------------------------------------------------------------------------------ grid barrier
+// The arrival counter is never cleared between launches (a memset node in front of every launch of a
+// block's chain cost ~2 us each): a launch starts from the count that the launch before it left in
+// bar[BAR_BASE], which CTA 0 moves on after the last barrier, when every CTA has read it.
 
 __device__ __forceinline__ void grid_barrier(unsigned* counter, unsigned& target, unsigned G, volatile int* err,
                                              unsigned limit = SPIN_LIMIT_GRID) {
@@ -701,7 +706,7 @@ __device__ __forceinline__ void grid_barrier(unsigned* counter, unsigned& target
     target += G;
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
     unsigned it = 0;
-    while (ld_acquire(counter) < target) {
+    while ((int)(ld_acquire(counter) - target) < 0) {   // (the counter may wrap)
       if (++it > limit || ((it & 255u) == 0 && *err != DEV_OK)) {
         atomicCAS(const_cast<int*>(err), DEV_OK, DEV_TIMEOUT_GRID);
         break;

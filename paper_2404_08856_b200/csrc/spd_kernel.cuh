@@ -127,6 +127,8 @@ __global__ void __launch_bounds__(ENGINE_THREADS, 1) forward_kernel(const __grid
     // ---------------- compute warps
     Ring ring{0, 0u, a.nstage};
     unsigned bar_target = 0, xphase = 0, cphase = 0;
+    const bool bar_global = !gemm_only && a.cluster_ctas == 0;
+    if (bar_global && tid == 0) bar_target = __ldcg(a.bar + BAR_BASE);
     // all CTAs wait for each other: through global memory, or inside the cluster
     auto sync_grid = [&]() {
       if (a.cluster_ctas) cluster_barrier(&ctl->cbar, cphase, (unsigned)G, err);
@@ -258,6 +260,7 @@ __global__ void __launch_bounds__(ENGINE_THREADS, 1) forward_kernel(const __grid
         stamp();
       }
       if (cta == 0 && tid == 0) {
+        if (bar_global) __stcg(a.bar + BAR_BASE, bar_target);
         if (a.mode == MODE_VERIFY) st->t_verify1 = globaltimer();
         else if (a.mode == MODE_DRAFT) st->t_draft1 = globaltimer();
       }
