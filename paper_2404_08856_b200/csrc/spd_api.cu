@@ -13,6 +13,7 @@
 #include "spd_prefill.cuh"
 #include "spd_gemm.cuh"
 #include "spd_attn.cuh"
+#include "spd_skinny.cuh"
 #include "spd_warp.cuh"
 #include "spd_tree.cuh"
 #include "spd_batch.cuh"
@@ -489,6 +490,28 @@ int row_ctas(int n_sm, int rows, int V) {
   return C;
 }
 
+// Top-k / top-p truncation of `rows` rows: one CTA per row, which holds the row in shared memory next to the
+// digit histogram, large where it fits.
+constexpr size_t TRUNC_ROOM = 6296;      // shared memory kept free of the row (with 256 bins the kernel declares 3 KB)
+bool trunc_fits(int V, int smem_optin) { return (size_t)V * sizeof(float) + TRUNC_ROOM <= (size_t)smem_optin; }
+cudaError_t launch_truncate(const float* in, float* out, int rows, int V, int top_k, float top_p, int smem_optin, cudaStream_t stream) {
+  static int attr[MAX_DEV][2];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess || dev < 0 || dev >= MAX_DEV) return e != cudaSuccess ? e : cudaErrorInvalidDevice;
+  const int smem = V * (int)sizeof(float);
+  auto go = [&](auto kernel, int slot) {
+    if (attr[dev][slot] < smem) {
+      const cudaError_t r = cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      if (r != cudaSuccess) return r;
+      attr[dev][slot] = smem;
+    }
+    kernel<<<rows, TRUNC_THREADS, smem, stream>>>(in, out, V, top_k, top_p);
+    return cudaGetLastError();
+  };
+  return (size_t)smem + TRUNC_BINS * 8 + 1024 <= (size_t)smem_optin ? go(truncate_rows_kernel<TRUNC_BINS>, 0) : go(truncate_rows_kernel<TRUNC_BINS_MIN>, 1);
+}
+
 // grid = CTAs of the launch; cluster > 0: they form one thread-block cluster (then grid == cluster)
 // and synchronise inside it, otherwise it is a cooperative launch with the barrier word `bar`.
 spd_status launch_forward(spd_ctx* ctx, int M, int dtype, StepArgs a, cudaStream_t stream, int grid, int cluster,
@@ -523,8 +546,8 @@ spd_status launch_forward(spd_ctx* ctx, int M, int dtype, StepArgs a, cudaStream
       // top-k / top-p: probability rows -> truncated and renormalised in place -> the rule on rows
       const int nrows = a.mode == MODE_VERIFY ? a.gamma + 1 : 1;
       prob_rows_kernel<<<n_sm_sampling, PROB_THREADS, 0, stream>>>(a, ctx->prow);
-      truncate_rows_kernel<<<nrows, WARP_THREADS, (size_t)a.md.V * sizeof(float), stream>>>(
-          ctx->prow, ctx->prow, a.md.V, ctx->cfg.top_k, ctx->cfg.top_p > 0.f ? ctx->cfg.top_p : 1.0f);
+      CU(launch_truncate(ctx->prow, ctx->prow, nrows, a.md.V, ctx->cfg.top_k, ctx->cfg.top_p > 0.f ? ctx->cfg.top_p : 1.0f,
+                         ctx->smem_optin, stream));
       CU(launch_rows(sample_rows_kernel, 1, C, ROW_THREADS, stream, false, a, C, ctx->prow));
     } else {
       CU(launch_rows(sample_step_kernel, 1, C, ROW_THREADS, stream, false, a, C));
@@ -879,11 +902,8 @@ spd_status alloc_ctx_buffers(spd_ctx* ctx) {
   if (ctx->truncate) {
     if ((s = dalloc(ctx, &ctx->prow, (size_t)MAX_M * V))) return s;
     // one CTA holds a whole row in shared memory
-    if ((size_t)V * sizeof(float) + sizeof(TruncScratch) + 1024 > (size_t)ctx->smem_optin)
+    if (!trunc_fits(V, ctx->smem_optin))
       return fail(ctx, SPD_EINVAL, "top-k / top-p: a vocabulary row does not fit the shared memory of one CTA");
-    if (cudaFuncSetAttribute((const void*)truncate_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)((size_t)V * sizeof(float))) != cudaSuccess)
-      return fail(ctx, SPD_ECUDA, "cannot size the truncation kernel's shared memory");
   }
   if ((s = dalloc(ctx, &ctx->rows, (size_t)cfg->max_seq * dmax))) return s;
   if ((s = dalloc(ctx, &ctx->ids_dev, (size_t)cfg->max_seq))) return s;
@@ -1332,8 +1352,8 @@ static spd_status tree_shape_from_parent(spd_ctx* ctx, int n, const int32_t* par
 static spd_status tree_prob_rows(spd_ctx* ctx, const StepArgs& a, cudaStream_t stream) {
   prob_rows_kernel<<<ctx->n_sm, PROB_THREADS, 0, stream>>>(a, ctx->prow);
   if (ctx->truncate)
-    truncate_rows_kernel<<<a.stat_n, WARP_THREADS, (size_t)a.md.V * sizeof(float), stream>>>(
-        ctx->prow, ctx->prow, a.md.V, ctx->cfg.top_k, ctx->cfg.top_p > 0.f ? ctx->cfg.top_p : 1.0f);
+    CU(launch_truncate(ctx->prow, ctx->prow, a.stat_n, a.md.V, ctx->cfg.top_k, ctx->cfg.top_p > 0.f ? ctx->cfg.top_p : 1.0f,
+                       ctx->smem_optin, stream));
   CU(cudaGetLastError());
   return SPD_OK;
 }
@@ -1603,8 +1623,8 @@ spd_status batch_probs(spd_batch* bt, int rows, int first, int stride) {
   CU(launch_rows(batch_softmax_kernel, rows, 1, ROW_THREADS, ctx->stream, true, bt->logits, first, stride, V, ctx->cfg.temperature, bt->stats,
                  ctx->truncate ? bt->probs : nullptr));
   if (ctx->truncate)
-    truncate_rows_kernel<<<rows, WARP_THREADS, (size_t)V * sizeof(float), ctx->stream>>>(
-        bt->probs, bt->probs, V, ctx->cfg.top_k, ctx->cfg.top_p > 0.f ? ctx->cfg.top_p : 1.0f);
+    CU(launch_truncate(bt->probs, bt->probs, rows, V, ctx->cfg.top_k, ctx->cfg.top_p > 0.f ? ctx->cfg.top_p : 1.0f, ctx->smem_optin,
+                       ctx->stream));
   CU(cudaGetLastError());
   return SPD_OK;
 }
@@ -1734,10 +1754,6 @@ spd_status spd_batch_create(spd_ctx* const* seqs, int B, spd_batch** out) {
   if (!s) s = balloc(bt, &bt->part_o, po * 8);
   if (!s) s = balloc(bt, &bt->part_ml, pu * 16);
   if (!s) s = balloc(bt, &bt->attn_cnt, ph);
-  if (!s && ctx->truncate &&
-      cudaFuncSetAttribute((const void*)truncate_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)((size_t)V * sizeof(float))) != cudaSuccess)
-    s = fail(ctx, SPD_ECUDA, "cannot size the truncation kernel's shared memory");
   if (s) { spd_batch_destroy(bt); return s; }
   *out = bt;
   return SPD_OK;
@@ -2051,23 +2067,17 @@ spd_status spd_truncate_probs(const float* probs, float* out, int rows, int V, i
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
     return SPD_ECUDA;
-  const size_t smem = (size_t)V * sizeof(float);
-  if (smem + sizeof(TruncScratch) + 1024 > (size_t)optin) {
+  if (!trunc_fits(V, optin)) {
     fprintf(stderr, "spd_truncate_probs: a row of %d probabilities does not fit shared memory\n", V);
     return SPD_EINVAL;
   }
-  if (cudaFuncSetAttribute((const void*)truncate_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-      cudaSuccess)
-    return SPD_ECUDA;
-  truncate_rows_kernel<<<rows, WARP_THREADS, smem, static_cast<cudaStream_t>(stream)>>>(probs, out, V, top_k, top_p);
-  return cudaGetLastError() == cudaSuccess ? SPD_OK : SPD_ECUDA;
+  return launch_truncate(probs, out, rows, V, top_k, top_p, optin, static_cast<cudaStream_t>(stream)) == cudaSuccess ? SPD_OK : SPD_ECUDA;
 }
 
-// Scratch of the two stand-alone GEMM entry points, per device: a status
-// block (DevState: only its error word is used) and, for spd_skinny_gemm, the tile-packed copy of w.
+// State of the two stand-alone GEMM entry points, per device: a status block (DevState: only its error word is
+// used) and, where the activations do not fit shared memory, the tile-packed copy of w.
 struct GemmScratch {
   bool ready = false;
-  unsigned* bar = nullptr;
   DevState* st = nullptr;
   char* packed = nullptr;
   size_t packed_cap = 0;
@@ -2075,6 +2085,45 @@ struct GemmScratch {
 };
 static GemmScratch g_gemm_scratch[MAX_DEV];      // spd_skinny_gemm (allocated on first use)
 static GemmScratch g_noalloc_state[MAX_DEV];     // spd_skinny_gemm_noalloc (points into g_noalloc_scratch)
+
+// The direct kernels (spd_skinny.cuh) take every shape whose activations fit a CTA's shared memory.
+static bool skinny_direct(int M, int K, size_t esz) { return sk_x_bytes(M, K, (int)esz) <= SK_X_MAX; }
+
+static spd_status launch_skinny(const float* x, const void* w, int dtype, int M, int N, int K, float* y, int n_sm, int* clear,
+                                cudaStream_t stream) {
+  const int esz = dtype == 1 ? 2 : 4, KB = sk_kb(K, esz);
+  // warps that share a tile: a warp keeps at least 4 (bf16, 64 bytes of a row each) or 2 (fp32, 512 bytes)
+  // K blocks, so that short rows are not cut into more pieces than there is latency to hide
+  int KS = SK_WARPS;
+  while (KS > 1 && KB < (dtype == 1 ? 4 : 2) * KS) KS >>= 1;
+  const size_t smem = SK_RED + (size_t)sk_x_bytes(M, K, esz);
+  const int groups = SK_WARPS / KS;
+  const int grid = (N + groups - 1) / groups < n_sm ? (N + groups - 1) / groups : n_sm;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEV) return SPD_ECUDA;
+  static bool attr[MAX_DEV][MAX_M + 1];
+  auto go = [&](auto kernel, int slot, auto... args) -> spd_status {
+    if (!attr[dev][slot]) {
+      if (cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SK_RED + SK_X_MAX) != cudaSuccess)
+        return SPD_ECUDA;
+      attr[dev][slot] = true;
+    }
+    kernel<<<grid, SK_THREADS, smem, stream>>>(args...);
+    return cudaGetLastError() == cudaSuccess ? SPD_OK : SPD_ECUDA;
+  };
+  if (dtype == 1) return go(skinny_bf16_kernel, 0, x, static_cast<const __nv_bfloat16*>(w), M, N, K, y, KS, clear);
+  const float* wf = static_cast<const float*>(w);
+  switch (M) {
+    case 1: return go(skinny_f32_kernel<1>, 1, x, wf, N, K, y, KS, clear);
+    case 2: return go(skinny_f32_kernel<2>, 2, x, wf, N, K, y, KS, clear);
+    case 3: return go(skinny_f32_kernel<3>, 3, x, wf, N, K, y, KS, clear);
+    case 4: return go(skinny_f32_kernel<4>, 4, x, wf, N, K, y, KS, clear);
+    case 5: return go(skinny_f32_kernel<5>, 5, x, wf, N, K, y, KS, clear);
+    case 6: return go(skinny_f32_kernel<6>, 6, x, wf, N, K, y, KS, clear);
+    case 7: return go(skinny_f32_kernel<7>, 7, x, wf, N, K, y, KS, clear);
+    default: return go(skinny_f32_kernel<8>, 8, x, wf, N, K, y, KS, clear);
+  }
+}
 
 spd_status spd_skinny_gemm(const float* x, const void* w, int dtype, int M, int N, int K, float* y, void* stream) {
   if (!x || !w || !y || M < 1 || M > MAX_M || N < 1 || K < 8 || K % 8 || (dtype != 0 && dtype != 1)) return SPD_EINVAL;
@@ -2087,17 +2136,16 @@ spd_status spd_skinny_gemm(const float* x, const void* w, int dtype, int M, int 
     cudaDeviceProp prop{};
     if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) return SPD_ECUDA;
     if (prop.major != 10) return SPD_ECUDA;
-    unsigned* bar = nullptr;
     DevState* st = nullptr;
-    if (cudaMalloc(&bar, 256) != cudaSuccess) return SPD_ENOMEM;
-    if (cudaMalloc(&st, sizeof(DevState)) != cudaSuccess) { cudaFree(bar); return SPD_ENOMEM; }
-    if (cudaMemset(st, 0, sizeof(DevState)) != cudaSuccess) { cudaFree(bar); cudaFree(st); return SPD_ECUDA; }
-    g.bar = bar; g.st = st;
+    if (cudaMalloc(&st, sizeof(DevState)) != cudaSuccess) return SPD_ENOMEM;
+    if (cudaMemset(st, 0, sizeof(DevState)) != cudaSuccess) { cudaFree(st); return SPD_ECUDA; }
+    g.st = st;
     g.n_sm = prop.multiProcessorCount;
     g.smem_optin = (int)prop.sharedMemPerBlockOptin;
     g.ready = true;   // only now: a failed set-up is repeated by the next call
   }
   const size_t esz = dtype == 1 ? 2 : 4;
+  if (skinny_direct(M, K, esz)) return launch_skinny(x, w, dtype, M, N, K, y, g.n_sm, nullptr, cs);
   const size_t need = packed_bytes(N, K, esz);
   if (need > g.packed_cap) {
     cudaStreamSynchronize(cs);
@@ -2112,7 +2160,7 @@ spd_status spd_skinny_gemm(const float* x, const void* w, int dtype, int M, int 
   a.mode = MODE_GEMM;
   a.st = g.st;
   a.gx = x; a.gw = g.packed; a.gy = y; a.gN = N; a.gK = K;
-  return launch_forward(ctx, M, dtype, a, cs, g.n_sm, 0, g.smem_optin, g.bar, g.n_sm);
+  return launch_forward(ctx, M, dtype, a, cs, g.n_sm, 0, g.smem_optin, nullptr, g.n_sm);
 }
 
 spd_status spd_skinny_gemm_status(int noalloc, void* stream) {
@@ -2152,7 +2200,6 @@ spd_status spd_skinny_gemm_noalloc(const float* x, const void* w, int dtype, int
     if (cudaGetSymbolAddress((void**)&ptr, g_noalloc_scratch) != cudaSuccess || !ptr) return SPD_ECUDA;
     g.n_sm = prop.multiProcessorCount;
     g.smem_optin = (int)prop.sharedMemPerBlockOptin;
-    g.bar = reinterpret_cast<unsigned*>(ptr);
     g.st = reinterpret_cast<DevState*>(ptr + 256);
     g.packed = reinterpret_cast<char*>(ptr + NOALLOC_HEADER);
     g.packed_cap = SPD_NOALLOC_MAX_PACKED_BYTES;
@@ -2160,7 +2207,9 @@ spd_status spd_skinny_gemm_noalloc(const float* x, const void* w, int dtype, int
   }
   spd_ctx* ctx = nullptr;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
-  // the array keeps whatever the last call left: the status block must start at zero
+  // the array keeps whatever the last call left: the status block must start at zero (the direct kernel
+  // clears its error word itself)
+  if (skinny_direct(M, K, esz)) return launch_skinny(x, w, dtype, M, N, K, y, g.n_sm, &g.st->err, cs);
   if (cudaMemsetAsync(g.st, 0, 256, cs) != cudaSuccess) return SPD_ECUDA;
   spd_status s = pack_tiles(ctx, g.packed, w, N, K, esz, g.n_sm, cs);
   if (s) return s;
@@ -2168,7 +2217,7 @@ spd_status spd_skinny_gemm_noalloc(const float* x, const void* w, int dtype, int
   a.mode = MODE_GEMM;
   a.st = g.st;
   a.gx = x; a.gw = g.packed; a.gy = y; a.gN = N; a.gK = K;
-  return launch_forward(ctx, M, dtype, a, cs, g.n_sm, 0, g.smem_optin, g.bar, g.n_sm);
+  return launch_forward(ctx, M, dtype, a, cs, g.n_sm, 0, g.smem_optin, nullptr, g.n_sm);
 }
 
 spd_status spd_wait_selftest(spd_ctx* ctx, int which, unsigned polls) {
