@@ -505,7 +505,7 @@ def run_gpu(args, rank, world):
                     "ms_per_step": ms_e2e / steps},
             # per block: gamma draft steps + one verify step, each one forward kernel (plus the two
             # sampling kernels behind it when not greedy)
-            "gpu_launches": (GAMMA + 1) * steps * (1 if greedy else 3),
+            "gpu_launches": (GAMMA + 1) * steps * (1 if greedy else 2),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                          "traffic": (VERIFY_TRAFFIC_RATIO * bytes_step if VERIFY_TRAFFIC_RATIO and GAMMA == 5 else None),
                          "traffic_source": "ncu capture on the 2-layer truncation, scaled by algorithmic bytes",

@@ -9,7 +9,7 @@
 //
 // What bounds it: MMA issue (two products, each twice for hi and lo: 4 x R^2 / 2 x d_head x 2 flops per
 // head).  640 rows, 32 heads x 128: three launches through fp32 scores in HBM took 36 + 54 + 24 us a
-// layer, this one 31; 1600 rows: 118 + ... -> see the launch list.
+// layer, this one 39.
 #pragma once
 #include "spd_engine.cuh"
 
