@@ -1,0 +1,112 @@
+"""Edges of the tiles and dispatch rules of the kernels: sizes around a tile, a warp, a cluster, the switch from
+one kernel to another, and the smallest ones, against the oracle or a 64-bit product.
+
+Tolerances.  Activations travel as bf16 hi + lo: x - (hi + lo) is at most 2^-17 |x|; products are accumulated in
+fp32 with fewer than 2^5 x 2^3 additions in a row per lane, warp and tile, so an element of X W^T is off by at
+most (2^-17 + 2^8 2^-24) sum |x| |w|: 2^-15 of that sum bounds it.  fp32 weights: 2^-17 of the same sum.
+Counts, tokens and truncated rows are exact.
+"""
+import numpy as np
+import pytest
+
+import synth
+from oracle import adapter as OA
+from oracle import sampling as S
+from oracle import warp
+
+from test_gpu_adapter import _run, _tiny_ctx
+from test_gpu_spd import _lib, lockstep
+from test_gpu_truncate import _dev_truncate
+
+F32 = np.float32
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,N,K,dtype", [
+    (1, 1, 8, 1), (2, 15, 24, 1), (3, 17, 32, 1), (8, 147, 40, 1), (5, 149, 1000, 1), (7, 2369, 2048, 1),
+    (6, 297, 6144, 1), (6, 297, 6152, 1),          # the last K whose fragments fit shared memory, the first that does not
+    (1, 1, 8, 0), (2, 3, 120, 0), (8, 5, 128, 0), (7, 150, 136, 0), (4, 593, 2056, 0),
+    (8, 33, 6144, 0), (8, 33, 6152, 0), (3, 64, 16384, 0)])
+@pytest.mark.parametrize("noalloc", [False, True])
+def test_skinny_gemm_edges(M, N, K, dtype, noalloc):
+    import torch
+    spd = _lib()
+    g = np.random.default_rng(M * 100000 + N * 10 + dtype)
+    x = g.standard_normal((M, K)).astype(F32)
+    w = (g.standard_normal((N, K)) * 0.05).astype(F32)
+    wd = torch.from_numpy(w).cuda()
+    if dtype == 1:
+        bits = synth.f32_to_bf16_bits(w)
+        w, wd = synth.bf16_bits_to_f32(bits), torch.from_numpy(bits.view(np.int16)).cuda()
+    y = torch.full((M, N), float("nan"), device="cuda")
+    (spd.skinny_gemm_noalloc if noalloc else spd.skinny_gemm)(torch.from_numpy(x).cuda(), wd, y, dtype)
+    torch.cuda.synchronize()
+    want = x.astype(np.float64) @ w.astype(np.float64).T
+    bound = np.abs(x).astype(np.float64) @ np.abs(w).astype(np.float64).T * 2.0 ** (-15 if dtype else -17)
+    got = y.cpu().numpy()
+    assert np.isfinite(got).all() and (np.abs(got - want) <= bound).all()
+    assert spd.skinny_gemm_status(noalloc) == 0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("B,gamma,V", [(1, 0, 1), (3, 1, 31), (2, 9, 1024), (20, 7, 4099), (75, 2, 8200), (149, 17, 700), (1, 5, 40000)])
+def test_rejection_rule_edges(B, gamma, V):
+    """Every cluster width, more rows than are taken together when greedy, vocabularies around a warp's piece."""
+    import torch
+    spd = _lib()
+    tl, dl = synth.microbench_logits(B, max(gamma, 1), V, 0.3)
+    p = S.softmax_t(np.ascontiguousarray(tl[:, :gamma + 1]), 1.0)
+    q = S.softmax_t(np.ascontiguousarray(dl[:, :gamma]), 1.0) if gamma else np.zeros((B, 0, V), F32)
+    for greedy in (False, True):
+        ids = (p[:, :gamma] if greedy else q).argmax(-1).astype(np.int32).reshape(B, gamma)
+        if greedy and gamma > 8:
+            ids[::2, 8] = (ids[::2, 8] + 1) % V        # a mismatch in the second group of rows
+        u = synth.uniforms(9, f"edge.{B}.{V}", (B, gamma + 1))
+        want_a, want_n = S.reject_sample_batch(p, q, ids, u, greedy)
+        a, n = (torch.full((B,), -7, dtype=torch.int32, device="cuda") for _ in range(2))
+        dev = [torch.from_numpy(np.ascontiguousarray(t)).cuda() if t.size else torch.zeros(1, device="cuda").to(torch.int32 if t is ids else torch.float32)
+               for t in (p, q, ids, u)]
+        spd.reject_sample(*dev, gamma, greedy, a, n)
+        assert np.array_equal(a.cpu().numpy(), want_a) and np.array_equal(n.cpu().numpy(), want_n)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("V", [1023, 1025, 32768, 53700, 56500])     # the last two: many and few digit bins fit beside the row
+def test_truncation_edges(V):
+    spd = _lib()
+    g = np.random.default_rng(V)
+    raw = np.floor(g.standard_exponential((3, V)) * 6).astype(F32)
+    raw[:, V // 2] += 1
+    rows = (raw / raw.sum(axis=1, keepdims=True)).astype(F32)
+    rows[1] = S.softmax_t(g.standard_normal((1, V)).astype(F32) * 3, 1.0)[0]
+    for top_k, top_p in [(1, 1.0), (V - 1, 0.5), (50, 0.9), (0, 0.9999)]:
+        want = warp.warp_rows(rows, top_k, top_p)
+        assert np.array_equal(_dev_truncate(spd, rows, top_k, top_p).view(np.uint32), want.view(np.uint32)), (top_k, top_p)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("m,d_in,d_hid,d_out", [(15, 64, 136, 128), (17, 72, 264, 257), (31, 128, 120, 1), (129, 200, 512, 130),
+                                               (257, 256, 256, 384), (513, 1024, 2312, 256)])
+def test_image_adapter_edges(m, d_in, d_hid, d_out):
+    """Row counts around the activation tiles (multiples of 16, 32 and 256), ragged widths, one and several K blocks;
+    the bound is the one of the adapter's own test."""
+    _lib()
+    gpu = _tiny_ctx()
+    feats = synth.vision_features(2, m, d_in)
+    w1, w2 = synth.adapter_mlp(1, "target", d_in, d_hid, d_out, std=0.05)
+    want = OA.image_adapter(feats, synth.bf16_bits_to_f32(w1), synth.bf16_bits_to_f32(w2))
+    got = _run(gpu, feats, w1, w2, False)
+    assert np.isfinite(got).all() and (np.abs(got - want) <= 1e-4 + 1e-4 * np.abs(want)).all()
+    gpu.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_image,n_prompt", [(0, 1), (0, 63), (1, 64), (64, 65), (100, 157)])
+@pytest.mark.parametrize("d_draft,heads", [(128, 2), (256, 2)])
+def test_prompt_lengths_around_the_attention_tiles(n_image, n_prompt, d_draft, heads):
+    """Prefill attention (64-row tiles, heads of 64 and 128) in lock-step with the oracle; the logit bound is that of
+    the other small bf16 models."""
+    t = synth.ModelCfg(1, 256, 2, 264, 1000, False, dtype="bf16")
+    d = synth.ModelCfg(2, d_draft, heads, 344, 1000, True, dtype="bf16")
+    wl = synth.Workload("edge", t, d, n_image, n_prompt, 4, 16)
+    assert lockstep(wl, False, 1.0, 2, 2e-2, std=0.08)["blocks"] == 2
