@@ -79,7 +79,6 @@ struct spd_ctx {
     __nv_bfloat16 *h_hi = nullptr, *h_lo = nullptr, *q_hi = nullptr, *q_lo = nullptr;
     __nv_bfloat16 *g_hi = nullptr, *g_lo = nullptr;   // silu(gate) * up [rows][d_ffn]
     float* wide = nullptr;                            // projection results, K slice by K slice
-    size_t cap_wide = 0;
   } pf;
   // scratch of spd_image_adapter, grown on demand
   struct {
@@ -803,9 +802,18 @@ __global__ void gather_rows_kernel(const int* ids, const float* table, float* ou
   }
 }
 
-// Most K slices of a projection whose reader adds them up, and the rows up to which that is offered
-// (their partial products then fit the widest activation buffer).
+// Most K slices of a projection whose reader adds them up.
 constexpr int UG_SLICES_MAX = 8;
+
+// Elements of the buffer that takes a projection's partial products in a call of R rows: whole sums of any
+// number of rows, all UG_SLICES_MAX slices of a batched step's.
+size_t wide_elems(const spd_ctx* ctx, int R) {
+  const spd_model_cfg &t = ctx->cfg.target, &d = ctx->cfg.draft;
+  const size_t dm = t.d_model > d.d_model ? t.d_model : d.d_model, ad = ctx->cfg.draft_adapter_in;
+  const size_t rp = ((size_t)R + 63) / 64 * 64, least = (size_t)UG_SLICES_MAX * BATCH_ROWS_MAX * 3 * dm;
+  const size_t whole = rp * (3 * dm > ad ? 3 * dm : ad);
+  return whole > least ? whole : least;
+}
 
 spd_status prefill_scratch(spd_ctx* ctx, int R) {
   if ((size_t)R <= ctx->pf.cap_rows) return SPD_OK;
@@ -816,24 +824,22 @@ spd_status prefill_scratch(spd_ctx* ctx, int R) {
   size_t kin = dm > fm ? dm : fm;
   if (ad > kin) kin = ad;
   const size_t rp = ((size_t)R + 63) / 64 * 64;
-  size_t wide = rp * (3 * dm > ad ? 3 * dm : ad);
-  if (wide < (size_t)UG_SLICES_MAX * BATCH_ROWS_MAX * 3 * dm) wide = (size_t)UG_SLICES_MAX * BATCH_ROWS_MAX * 3 * dm;
   spd_status s;   // earlier buffers stay in the context's allocation list until spd_destroy
   if ((s = dalloc(ctx, &ctx->pf.h_hi, rp * kin))) return s;
   if ((s = dalloc(ctx, &ctx->pf.h_lo, rp * kin))) return s;
   if ((s = dalloc(ctx, &ctx->pf.q_hi, rp * dm))) return s;
   if ((s = dalloc(ctx, &ctx->pf.q_lo, rp * dm))) return s;
-  if ((s = dalloc(ctx, &ctx->pf.wide, wide))) return s;
+  if ((s = dalloc(ctx, &ctx->pf.wide, wide_elems(ctx, R)))) return s;
   if ((s = dalloc(ctx, &ctx->pf.g_hi, rp * fm))) return s;
   if ((s = dalloc(ctx, &ctx->pf.g_lo, rp * fm))) return s;
-  ctx->pf.cap_wide = wide;
   ctx->pf.cap_rows = rp;
   return SPD_OK;
 }
 
-// K slices that fit the activation buffer for an [R][N] result.
-int slices_that_fit(const spd_ctx* ctx, int R, int N) {
-  const size_t n = ctx->pf.cap_wide / ((size_t)R * N);
+// K slices of an [R][N] result that a call of `rows` rows has room for: a rule over the call's own size, not over
+// what earlier calls have made the buffer, so that a prompt is summed in the same order whatever came before it.
+int slices_that_fit(const spd_ctx* ctx, int rows, int R, int N) {
+  const size_t n = wide_elems(ctx, rows) / ((size_t)R * N);
   return n < 1 ? 1 : (n < UG_SLICES_MAX ? (int)n : UG_SLICES_MAX);
 }
 
@@ -852,11 +858,12 @@ spd_status launch_prefill_attn(spd_ctx* ctx, const __nv_bfloat16* kc, const __nv
 
 // Dense forward of rows X [R][d] (fp32, device; positions 0..R-1) through every layer of a
 // bf16 model: fills the KV cache rows 0..R-1 and leaves the final residual stream in X.  Seven launches
-// a layer; a projection whose reader can add K slices up is sliced where that fills the device.
-spd_status prefill_tc(spd_ctx* ctx, ModelHost& mh, float* X, int R) {
+// a layer; a projection whose reader can add K slices up is sliced where that fills the device.  `rows`: those
+// of the call's larger pass, which the buffers are sized for.
+spd_status prefill_tc(spd_ctx* ctx, ModelHost& mh, float* X, int R, int rows) {
   const int d = mh.cfg.d_model, f = mh.cfg.d_ffn, H = mh.cfg.n_heads, dh = d / H, L = mh.cfg.n_layers;
   spd_status s;
-  if ((s = prefill_scratch(ctx, R))) return s;
+  if ((s = prefill_scratch(ctx, rows))) return s;
   auto& pf = ctx->pf;
   cudaStream_t cs = ctx->stream;
   const size_t max_seq = ctx->cfg.max_seq, xs = (size_t)R * d;
@@ -869,17 +876,17 @@ spd_status prefill_tc(spd_ctx* ctx, ModelHost& mh, float* X, int R) {
     __nv_bfloat16* vc = static_cast<__nv_bfloat16*>(mh.md.vcache) + (size_t)l * max_seq * d;
     int sl = 1;
     if ((s = ug_gemm(ctx, pf.h_hi, pf.h_lo, R, d, w.wqkv, 3 * d, UG_F32, pf.wide, nullptr, nullptr, 3 * d,
-                     slices_that_fit(ctx, R, 3 * d), &sl))) return s;
+                     slices_that_fit(ctx, rows, R, 3 * d), &sl))) return s;
     CU(launch_dependent(rope_kv_kernel, dim3(rope_blocks), dim3(256), 0, cs, pf.wide, sl, R, d, dh, mh.md.rope_cos, mh.md.rope_sin,
                         pf.q_hi, pf.q_lo, kc, vc, (int)max_seq));
     if ((s = dh == 128 ? launch_prefill_attn<128>(ctx, kc, vc, R, H, mh.md.scale) : launch_prefill_attn<64>(ctx, kc, vc, R, H, mh.md.scale)))
       return s;
-    if ((s = ug_gemm(ctx, pf.h_hi, pf.h_lo, R, d, w.wo, d, UG_F32, pf.wide, nullptr, nullptr, d, slices_that_fit(ctx, R, d), &sl))) return s;
+    if ((s = ug_gemm(ctx, pf.h_hi, pf.h_lo, R, d, w.wo, d, UG_F32, pf.wide, nullptr, nullptr, d, slices_that_fit(ctx, rows, R, d), &sl))) return s;
     CU(launch_dependent(resid_rms_split_kernel, dim3(R), dim3(256), 0, cs, X, pf.wide, sl, xs, w.ffn_norm, mh.cfg.rms_eps, d, pf.h_hi,
                         pf.h_lo));
     // gate/up with SwiGLU in the epilogue (interleaved gate/up rows): hi/lo [R][f] straight out of the GEMM
     if ((s = ug_gemm(ctx, pf.h_hi, pf.h_lo, R, d, w.wgu, 2 * f, UG_SWIGLU, nullptr, pf.g_hi, pf.g_lo, f))) return s;
-    if ((s = ug_gemm(ctx, pf.g_hi, pf.g_lo, R, f, w.wd, d, UG_F32, pf.wide, nullptr, nullptr, d, slices_that_fit(ctx, R, d), &sl))) return s;
+    if ((s = ug_gemm(ctx, pf.g_hi, pf.g_lo, R, f, w.wd, d, UG_F32, pf.wide, nullptr, nullptr, d, slices_that_fit(ctx, rows, R, d), &sl))) return s;
     // the norm in front of the next layer rides on the residual update
     CU(launch_dependent(resid_rms_split_kernel, dim3(R), dim3(256), 0, cs, X, pf.wide, sl, xs,
                         l + 1 < L ? mh.rm[l + 1].attn_norm : mh.md.final_norm, mh.cfg.rms_eps, d, pf.h_hi, pf.h_lo));
@@ -1107,8 +1114,8 @@ spd_status spd_prefill(spd_ctx* ctx, const float* image_embeds, int m, const flo
   if (use_tc_prefill(dm) && use_tc_prefill(tm)) {
     // ---- dense tensor-core pass over all rows of each model
     const int dd = dm.cfg.d_model, dt = tm.cfg.d_model;
-    const int Rd = (ad > 0 ? m : 0) + n, Rt = m + n;
-    if ((s = prefill_scratch(ctx, Rt > Rd ? Rt : Rd))) return s;
+    const int Rd = (ad > 0 ? m : 0) + n, Rt = m + n, rows = Rt > Rd ? Rt : Rd;
+    if ((s = prefill_scratch(ctx, rows))) return s;
     float* X = ctx->rows;
     dm.pos_base = 0;
     if (ad > 0 && dm.rows_given) {   // draft rows [given image rows ; embed(prompt)]
@@ -1123,13 +1130,13 @@ spd_status spd_prefill(spd_ctx* ctx, const float* image_embeds, int m, const flo
     }
     gather_rows_kernel<<<592, 256, 0, ctx->stream>>>(ctx->ids_dev, dm.md.embed, X + (size_t)dm.pos_base * dd, n, dd, V,
                                                        &ctx->st->err);
-    if ((s = prefill_tc(ctx, dm, X, Rd))) return s;
+    if ((s = prefill_tc(ctx, dm, X, Rd, rows))) return s;
     // ---- target rows [V_1..V_m ; embed(prompt)] (Eq. 1); last row -> first generated token
     tm.pos_base = m;
     if (m > 0)
       CU(cudaMemcpyAsync(X, image_embeds, (size_t)m * dt * sizeof(float), cudaMemcpyDefault, ctx->stream));
     gather_rows_kernel<<<592, 256, 0, ctx->stream>>>(ctx->ids_dev, tm.md.embed, X + (size_t)m * dt, n, dt, V, &ctx->st->err);
-    if ((s = prefill_tc(ctx, tm, X, Rt))) return s;
+    if ((s = prefill_tc(ctx, tm, X, Rt, rows))) return s;
     CU(cudaMemcpyAsync(tm.md.x, X + (size_t)(Rt - 1) * dt, dt * sizeof(float), cudaMemcpyDeviceToDevice, ctx->stream));
     StepArgs a = base_args(ctx, tm);
     a.mode = MODE_ROWS; a.skip_layers = 1; a.want_sample = 1;

@@ -14,6 +14,8 @@ from oracle import adapter as OA
 from oracle import sampling as S
 from oracle import warp
 
+import harness as H
+
 from test_gpu_adapter import _run, _tiny_ctx
 from test_gpu_spd import _lib, lockstep
 from test_gpu_truncate import _dev_truncate
@@ -110,3 +112,30 @@ def test_prompt_lengths_around_the_attention_tiles(n_image, n_prompt, d_draft, h
     d = synth.ModelCfg(2, d_draft, heads, 344, 1000, True, dtype="bf16")
     wl = synth.Workload("edge", t, d, n_image, n_prompt, 4, 16)
     assert lockstep(wl, False, 1.0, 2, 2e-2, std=0.08)["blocks"] == 2
+
+
+@pytest.mark.gpu
+def test_a_prompt_is_summed_in_the_same_order_whatever_came_before_it():
+    """540 rows of a 256-wide model: a length at which the room for K slices depends on the rows it is taken from.
+    Logits bit for bit on a fresh context, behind a longer prompt, and on a fork of the context that had it."""
+    _lib()
+    t = synth.ModelCfg(1, 256, 2, 264, 1000, False, dtype="bf16")
+    d = synth.ModelCfg(1, 128, 2, 344, 1000, True, dtype="bf16")
+    wl = synth.Workload("order", t, d, 0, 540, 4, 16)
+    tw, dw = H.build_weights(wl, 0.08)
+    gpu = H.make_gpu(wl, tw, dw, 2100, 1.0, True)
+    ids = synth.prompt_ids(wl)
+    longer = np.resize(ids, 2048).astype(np.int32)
+
+    def logits(ctx):
+        ctx.prefill(None, ids)
+        return ctx.get_logits(1).copy()
+
+    fresh = logits(gpu)
+    gpu.prefill(None, longer)
+    again, other = logits(gpu), gpu.fork()
+    forked = logits(other)
+    assert np.array_equal(fresh.view(np.uint32), again.view(np.uint32))
+    assert np.array_equal(fresh.view(np.uint32), forked.view(np.uint32))
+    other.close()
+    gpu.close()
