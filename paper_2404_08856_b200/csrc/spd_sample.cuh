@@ -152,6 +152,7 @@ __device__ bool row_pick(WF wf, int V, unsigned long long Z, float u, const RowS
     tok = sc->cidx[0];
     for (int c = 1; c < rs.C; ++c)
       if (sc->cmax[c] > m) { m = sc->cmax[c]; tok = sc->cidx[c]; }
+    if (tok >= V) tok = 0;      // a row of NaN has no largest weight
     return rs.rank == 0;
   }
   const unsigned long long T = threshold(Z, u);

@@ -139,3 +139,59 @@ def test_a_prompt_is_summed_in_the_same_order_whatever_came_before_it():
     assert np.array_equal(fresh.view(np.uint32), forked.view(np.uint32))
     other.close()
     gpu.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("V", [64, 1000, 4100, 32000])
+def test_draws_from_rows_that_are_no_distribution(V):
+    """Rows of NaN, of infinity and without any mass give a token of the vocabulary, in one CTA and across clusters.
+    A NaN counts 2^63, so an even number of them adds up to no mass (modulo 2^64): then the largest weight, lowest
+    index, of the entries that are numbers, and 0 if there is none."""
+    import torch
+    spd = _lib()
+    nan, inf = np.nan, np.inf
+    tiny = np.full(V, nan, F32)
+    tiny[[7, V - 3]] = [1e-12, 2e-12]
+    one = np.zeros(V, F32)
+    one[V - 5] = inf
+    flat = np.full(V, 1.0 / V, F32)
+    half = np.zeros(V, F32)            # target 1/2 of the draft everywhere: nothing is left after a rejection
+    half[: V // 2] = 1.0 / V
+    # (target row under test, draft row, u of the accept test, accepted, next)
+    rows = [(np.full(V, nan, F32), flat, 0.5, 1, 0), (tiny, flat, 0.5, 1, V - 3), (one, flat, 0.5, 1, V - 5), (half, 2 * half, 0.75, 0, 0)]
+    p = np.stack([np.stack([flat if a else t, t]) for t, _, _, a, _ in rows])
+    q = np.stack([d[None] for _, d, _, _, _ in rows])
+    u = np.array([[x, 0.25] for _, _, x, _, _ in rows], F32)
+    ids = np.zeros((len(rows), 1), np.int32)
+    a, n = (torch.full((len(rows),), -7, dtype=torch.int32, device="cuda") for _ in range(2))
+    dev = [torch.from_numpy(x).cuda() for x in (p, q, ids, u)]
+    spd.reject_sample(*dev, 1, False, a, n)
+    assert a.cpu().tolist() == [r[3] for r in rows] and n.cpu().tolist() == [r[4] for r in rows]
+    greedy = np.stack([np.full((2, V), x, F32) for x in (nan, -inf)] + [np.stack([one, one])])
+    ids = np.array([[0], [0], [V - 5]], np.int32)
+    spd.reject_sample(torch.from_numpy(greedy).cuda(), None, torch.from_numpy(ids).cuda(), None, 1, True, a[:3], n[:3])
+    assert a[:3].cpu().tolist() == [1, 1, 1] and n[:3].cpu().tolist() == [0, 0, V - 5]
+    trunc = np.stack([np.where(np.arange(V) % 3 == 1, F32(nan), flat), np.where(np.arange(V) % 2 == 0, -flat, flat)]).astype(F32)
+    want = warp.warp_rows(np.where(trunc > 0, trunc, F32(0)), 20, 0.9)
+    assert np.array_equal(_dev_truncate(spd, trunc, 20, 0.9).view(np.uint32), want.view(np.uint32))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+def test_a_step_whose_logits_are_nan_yields_a_token_of_the_vocabulary(dtype):
+    """NaN image rows make every logit of the target NaN: the first token and the one a verify step emits are 0."""
+    _lib()
+    t = synth.ModelCfg(2, 256, 4, 688, 1024, False, dtype=dtype)
+    d = synth.ModelCfg(1, 128, 2, 344, 1024, False, dtype=dtype)
+    wl = synth.Workload("nan", t, d, 16, 16, 4, 32)
+    tw, dw = H.build_weights(wl, 0.1)
+    gpu = H.make_gpu(wl, tw, dw, 96, 1.0, False)
+    img, ids = synth.image_embeds(wl), synth.prompt_ids(wl)
+    u = synth.uniforms(5, "nan", 8)
+    assert gpu.prefill(np.full_like(img, np.nan), ids, u0=0.5) == 0
+    gpu.draft(2, u[:2])
+    assert gpu.verify(2, u[2:5])[1] == 0
+    assert np.isnan(gpu.get_logits(3)).all()
+    gpu.draft(2, u[:2])                     # the next step takes the emitted token as it is
+    gpu.verify(2, u[2:5])
+    gpu.close()
