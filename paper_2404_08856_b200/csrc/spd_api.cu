@@ -580,6 +580,15 @@ spd_status sync_state(spd_ctx* ctx, cudaStream_t stream = nullptr, bool use_give
   return SPD_OK;
 }
 
+// Calls that set host-side bookkeeping for work that has to run exactly once (a replayed graph would move the
+// sequence without the host's bound on its length, or never upload what the host believes uploaded).
+spd_status refuse_capture(spd_ctx* ctx, const char* call) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  CU(cudaStreamIsCapturing(ctx->stream, &cap));
+  if (cap != cudaStreamCaptureStatusNone) return fail(ctx, SPD_ECUDA, std::string(call) + " cannot be captured into a graph");
+  return SPD_OK;
+}
+
 // Results that live in the device state.  Device destinations are copied on the stream at once; for host
 // destinations the caller reads the whole state back with one pinned copy (sync_state) and hands
 // them out with put_result: a copy per word into pageable memory would block for each.
@@ -1652,9 +1661,10 @@ spd_status batch_room(spd_batch* bt, int rows, bool draft) {
 template <class T>
 spd_status upload_changed(spd_ctx* ctx, T* dev, std::vector<T>& have, const std::vector<T>& now) {
   if (have.size() == now.size() && !memcmp(have.data(), now.data(), now.size() * sizeof(T))) return SPD_OK;
-  have = now;
-  CU(cudaMemcpyAsync(dev, have.data(), have.size() * sizeof(T), cudaMemcpyHostToDevice, ctx->stream));
+  have.clear();      // until the copy has landed the device's contents are not known
+  CU(cudaMemcpyAsync(dev, now.data(), now.size() * sizeof(T), cudaMemcpyHostToDevice, ctx->stream));
   CU(cudaStreamSynchronize(ctx->stream));
+  have = now;
   return SPD_OK;
 }
 
@@ -1780,6 +1790,7 @@ static spd_status batch_refresh(spd_batch* bt) {
     memcpy(&hd[b], &c->draft.md, sizeof(ModelDev));
   }
   spd_status s;
+  if ((s = refuse_capture(ctx, "a batched step"))) return s;
   if ((s = upload_changed(ctx, bt->seqs_dev, bt->h_seqs, hs))) return s;
   if ((s = upload_changed(ctx, bt->mds_t, bt->h_t, ht))) return s;
   return upload_changed(ctx, bt->mds_d, bt->h_d, hd);
@@ -2033,6 +2044,8 @@ spd_status spd_rollback(spd_ctx* ctx, int n_text, int32_t prev_token, int32_t pe
   if (n_text < 1 || ctx->m_image + n_text + 1 > ctx->cfg.max_seq || prev_token < 0 || prev_token >= V ||
       pending_token < 0 || pending_token >= V)
     return fail(ctx, SPD_EINVAL, "bad rollback arguments");
+  spd_status s = refuse_capture(ctx, "spd_rollback");
+  if (s) return s;
   // (three words by value: a copy from the host would have to wait for the stream)
   set_sequence_kernel<<<1, 1, 0, ctx->stream>>>(ctx->st, n_text, pending_token, prev_token);
   CU(cudaGetLastError());

@@ -195,3 +195,75 @@ def test_a_step_whose_logits_are_nan_yields_a_token_of_the_vocabulary(dtype):
     gpu.draft(2, u[:2])                     # the next step takes the emitted token as it is
     gpu.verify(2, u[2:5])
     gpu.close()
+
+
+def _small_bf16_on_a_stream(stream, greedy=True):
+    spd = _lib()
+    t = synth.ModelCfg(1, 256, 4, 344, 1024, False, dtype="bf16")
+    d = synth.ModelCfg(1, 128, 2, 344, 1024, False, dtype="bf16")
+    wl = synth.Workload("stream", t, d, 0, 16, 4, 16)
+    tw, dw = H.build_weights(wl, 0.15)
+    return spd, wl, spd.Spd(t, d, tw.stored, dw.stored, 96, 7, 1.0, greedy, stream=stream.cuda_stream)
+
+
+def _refused_while_capturing(spd, stream, call):
+    import torch
+    x = torch.zeros(8, device="cuda")
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        graph = torch.cuda.CUDAGraph()
+        graph.capture_begin()
+        try:
+            x.add_(1)
+            with pytest.raises(spd.SpdError) as e:
+                call()
+        finally:
+            graph.capture_end()
+    assert e.value.status == spd.SPD_ECUDA
+
+
+@pytest.mark.gpu
+def test_rollback_is_refused_while_the_stream_is_being_captured():
+    """The host's bound on the sequence length must not follow a rollback that may never run."""
+    import torch
+    stream = torch.cuda.Stream()
+    spd, wl, gpu = _small_bf16_on_a_stream(stream)
+    ids = synth.prompt_ids(wl)
+    first = gpu.prefill(None, ids)
+    want, _ = gpu.generate(8, 4)
+    at = gpu.get_state()
+    _refused_while_capturing(spd, stream, lambda: gpu.rollback(len(ids), int(ids[-1]), first))
+    assert gpu.get_state() == at
+    gpu.rollback(len(ids), int(ids[-1]), first)
+    got, _ = gpu.generate(8, 4)
+    assert np.array_equal(got, want)
+    gpu.close()
+
+
+@pytest.mark.gpu
+def test_batched_steps_are_refused_while_the_stream_is_being_captured():
+    """... neither on a batch that has never run, whose descriptors would not reach the device, nor on a used one."""
+    import torch
+    stream = torch.cuda.Stream()
+    spd, wl, gpu = _small_bf16_on_a_stream(stream)
+    ids = synth.prompt_ids(wl)
+    first = gpu.prefill(None, ids)
+    want, _ = gpu.generate(16, 3)
+    other = gpu.fork()
+    for c in (gpu, other):
+        c.prefill(None, ids)
+    bt = spd.SpdBatch([gpu, other])
+    got = [[first], [first]]
+    for _ in range(3):
+        _refused_while_capturing(spd, stream, lambda: bt.draft(3, read_ids=False))
+        d = bt.draft(3)
+        _refused_while_capturing(spd, stream, lambda: bt.verify(3, read=False))
+        a, n = bt.verify(3)
+        for k in range(2):
+            got[k] += [int(x) for x in d[k][: a[k]]] + [int(n[k])]
+    for k in range(2):
+        m = min(len(got[k]), 16)
+        assert got[k][:m] == want[:m].tolist()
+    bt.close()
+    other.close()
+    gpu.close()
