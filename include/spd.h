@@ -300,7 +300,8 @@ spd_status spd_batch_verify_bytes(spd_batch* batch, int gamma, double* bytes);
 
 /* Logits of the last spd_verify (rows <= gamma+1) / of the last spd_draft (rows <= gamma):
  * fp32 [rows, vocab] into host or device memory.  Prefill's last row: spd_get_logits with
- * rows = 1 directly after spd_prefill. */
+ * rows = 1 directly after spd_prefill.  The draft's rows share a buffer of eight with later calls: after an
+ * spd_generate or spd_draft_tree with r rows in its widest level (at least 2), 8 - r are left. */
 spd_status spd_get_logits(spd_ctx* ctx, float* logits, int rows);
 spd_status spd_get_draft_logits(spd_ctx* ctx, float* logits, int rows);
 

@@ -625,6 +625,12 @@ void geom_draft_step(StepArgs& a, int j) {
   a.stat_r0 = 1; a.stat_n = 1;
 }
 
+// A launch that leaves draft logits in rows [0, n): spd_draft keeps step j's row at 7 - j, so its later steps' rows
+// are gone.
+void draft_logits_below(spd_ctx* ctx, int n) {
+  if (ctx->last_draft_rows > MAX_M - n) ctx->last_draft_rows = MAX_M - n;
+}
+
 StepArgs base_args(spd_ctx* ctx, ModelHost& mh) {
   StepArgs a{};
   a.md = mh.md;
@@ -1276,7 +1282,7 @@ spd_status spd_draft(spd_ctx* ctx, int gamma, const float* uniforms, int32_t* dr
     if (s) return s;
   }
   ctx->drafted_gamma = gamma;
-  ctx->last_draft_rows = gamma < MAX_M - 2 ? gamma : MAX_M - 2;
+  ctx->last_draft_rows = gamma;
   bool need_sync = false;
   spd_status s;
   if (draft_probs && !ctx->cfg.greedy)
@@ -1406,6 +1412,7 @@ spd_status spd_draft_tree(spd_ctx* ctx, int depth, const int32_t* branching, con
   }
   if (uniforms) CU(cudaMemcpyAsync(ctx->ubuf, uniforms, n * sizeof(float), cudaMemcpyDefault, ctx->stream));
   ModelHost& dm = ctx->draft;
+  draft_logits_below(ctx, 2);
   for (int lev = 0; lev < depth; ++lev) {
     StepArgs a = base_args(ctx, dm);
     a.mode = MODE_DRAFT; a.gamma = n; a.j = lev; a.tree = 1;
@@ -1425,6 +1432,7 @@ spd_status spd_draft_tree(spd_ctx* ctx, int depth, const int32_t* branching, con
         }
       a.n_slots = n + 1;
       a.stat_r0 = 0; a.stat_n = M;
+      draft_logits_below(ctx, M);
     }
     if ((s = launch_model(ctx, dm, M, a, ctx->stream))) return s;
     a.fwd_grid = dm.grid; a.sample_r0 = M - 1;
@@ -1926,6 +1934,7 @@ spd_status spd_generate(spd_ctx* ctx, int n_new, int gamma, const float* uniform
     CU(cudaStreamSynchronize(ctx->stream));   // the blocks run on the internal stream
   }
   ModelHost &tm = ctx->target, &dm = ctx->draft;
+  if (gamma > 0) draft_logits_below(ctx, 2);
   double ms_d = 0.0, ms_v = 0.0;
   // One block = gamma draft launches + one verify launch.  Everything a block needs (lengths,
   // tokens, block counter, uniforms) lives on the device, so the same CUDA graph is replayed for

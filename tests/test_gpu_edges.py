@@ -267,3 +267,32 @@ def test_batched_steps_are_refused_while_the_stream_is_being_captured():
     bt.close()
     other.close()
     gpu.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+def test_draft_logits_of_every_step_are_kept(dtype):
+    """gamma = 7: all seven rows, whose softmax is the step's distribution (the same numbers but for the order of
+    one sum: 2^-18 of each); what a later call has written over is refused, the rest is unchanged."""
+    import torch
+    spd = _lib()
+    t = synth.ModelCfg(1, 256, 4, 344, 1024, False, dtype=dtype)
+    d = synth.ModelCfg(2, 128, 2, 344, 1024, False, dtype=dtype)
+    wl = synth.Workload("rows", t, d, 0, 16, 7, 16)
+    tw, dw = H.build_weights(wl, 0.1)
+    gpu = H.make_gpu(wl, tw, dw, 96, 1.0, False)
+    gpu.prefill(None, synth.prompt_ids(wl), u0=0.5)
+    u = synth.uniforms(3, "rows", 16)
+    probs = torch.zeros(7, 1024, device="cuda")
+    gpu.draft(7, u[:7], probs_out=probs)
+    rows = gpu.get_draft_logits(7)
+    want = probs.cpu().numpy()
+    assert (np.abs(S.softmax_t(rows, 1.0) - want) <= 2.0 ** -18 * want + 1e-12).all()
+    for branching, left in (([1, 1, 1], 6), ([4], 6), ([2, 2], 6), ([3, 1], 5)):
+        gpu.draft_tree(branching, u[:7])
+        for refused in range(left + 1, 8):
+            with pytest.raises(spd.SpdError) as e:
+                gpu.get_draft_logits(refused)
+            assert e.value.status == spd.SPD_EINVAL
+        assert np.array_equal(gpu.get_draft_logits(left).view(np.uint32), rows[:left].view(np.uint32))
+    gpu.close()
