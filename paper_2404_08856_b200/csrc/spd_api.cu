@@ -5,6 +5,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -481,12 +482,26 @@ cudaError_t launch_rows(void (*kernel)(KA...), int rows, int C, int threads, cud
   return cudaLaunchKernelEx(&cfg, kernel, KA(args)...);
 }
 
-// CTAs per row: as many as keep all rows on the device at once, at most 8 (the portable cluster size), and
-// none with less than ~1000 entries of the row (a CTA's fixed cost is then larger than its share).
+// CTAs per row.  Below ~6000 entries one: a cluster's launch and barrier cost more than its share of the row is worth.  Then
+// 4 and 8 (the portable cluster size), as long as all rows are on the device at once.  Device time of the rule on one /
+// 16 sequences, us, with 1, 4, 8 CTAs of 512 threads: 4000 entries 4.2, 5.0, 4.9 / 4.3, 5.2, 5.7; 6000 4.1, 4.8, 5.0 / 5.0, 5.3, 5.6;
+// 8000 5.5, 4.9, 5.0 / 5.7, 5.2, 6.2; 16000 8.9, 5.4, 5.1 / 9.2, 5.6, 6.1; 32000 8.1, 5.7, 5.1 / 13.4, 7.0, 5.9.  (2 CTAs are never the
+// best: 5.3 at 8000.)
 int row_ctas(int n_sm, int rows, int V) {
-  int C = ROW_CTAS_MAX;
-  while (C > 1 && (rows * C > n_sm || V / C < ROW_THREADS)) C >>= 1;
+  int C = V <= 6144 ? 1 : (V <= 16384 ? 4 : ROW_CTAS_MAX);
+  while (C > 1 && rows * C > n_sm) C >>= 1;
   return C;
+}
+
+// SMs of a device, asked for once.
+int device_sms(int dev) {
+  static std::atomic<int> known[MAX_DEV];
+  const bool kept = dev >= 0 && dev < MAX_DEV;
+  int n = kept ? known[dev].load(std::memory_order_relaxed) : 0;
+  if (n > 0) return n;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+  if (kept) known[dev].store(n, std::memory_order_relaxed);
+  return n;
 }
 
 // Top-k / top-p truncation of `rows` rows: one CTA per row, which holds the row in shared memory next to the
@@ -2078,13 +2093,18 @@ spd_status spd_reject_sample(const float* p, const float* q, const int32_t* ids,
   if (!p || !n_acc || !next || B < 1 || gamma < 0 || V < 1) return SPD_EINVAL;
   if (gamma > 0 && !ids) return SPD_EINVAL;
   if (!greedy && (!u || (gamma > 0 && !q))) return SPD_EINVAL;
-  int dev = 0, n_sm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return SPD_ECUDA;
-  // four entries of the row per thread: with a small vocabulary many sequences share an SM
-  const int C = row_ctas(n_sm, B, V);
-  int threads = ((V / C + 3) / 4 + 31) / 32 * 32;
-  if (threads > ROW_THREADS) threads = ROW_THREADS;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return SPD_ECUDA;
+  const int n_sm = device_sms(dev);
+  if (n_sm < 1) return SPD_ECUDA;
+  // four entries of a slice per thread up to 512 threads (with a small vocabulary many sequences share an SM), more than
+  // 512 only for slices of over 8000 entries: 32000 entries on 1 / 2 / 4 / 8 CTAs, 32 (8: 4) sequences, us: 512 threads 13.6 / 10.5 /
+  // 7.2 / 5.7, 1024 threads 10.9 / 8.3 / 6.8 / 6.7
+  // (greedy decoding mostly looks at more rows than one: clusters are worth it from shorter rows on, 6 accepted rows of 6000 on
+  // 1 / 4 CTAs 8.5 / 7.2 us, of 16000 on 4 / 8 CTAs 9.1 / 7.6)
+  const int C = row_ctas(n_sm, B, greedy ? V + V / 2 : V), slice = (V + C - 1) / C, most = slice > 8000 ? ROW_THREADS : ROW_THREADS / 2;
+  int threads = ((slice + 3) / 4 + 31) / 32 * 32;
+  if (threads > most) threads = most;
   return launch_rows(reject_sample_kernel, B, C, threads, static_cast<cudaStream_t>(stream), false, p, q, ids, u, gamma, V, greedy, C, n_acc,
                      next) == cudaSuccess ? SPD_OK : SPD_ECUDA;
 }

@@ -372,8 +372,8 @@ __global__ void __launch_bounds__(ROW_THREADS) batch_draft_sample_kernel(const B
     const RowStats st = probs ? RowStats{0.f, 1.f} : row_stats(lrow, V, temperature, rs, &ss);
     auto wf = [&](int k) { return prow ? ldcg(prow + k) : prob_of(ldcg(lrow + k), temperature, st.mx, st.sum); };
     float* q = q_all + ((size_t)b * gamma + j) * V;
-    const unsigned long long Z = row_mass(wf, [&](int k, float w) { stcg(q + k, w); }, V, rs, &sc);
-    mine = row_pick(wf, V, Z, u[(size_t)b * gamma + j], rs, &sc, tok);
+    const RowMass m = row_mass(wf, [&](int k, float w) { stcg(q + k, w); }, V, rs, &sc);
+    mine = row_pick(wf, V, m, u[(size_t)b * gamma + j], rs, &sc, tok);
   }
   if (mine && threadIdx.x == 0) {
     seqs[b].st->d_ids[j] = tok;

@@ -343,8 +343,8 @@ __global__ void __launch_bounds__(ROW_THREADS) sample_step_kernel(const __grid_c
     const float* lrow = a.logits + (size_t)r0 * V;
     float* qrow = a.q_out + (size_t)a.j * V;
     auto wf = [&](int k) { return prob_of(ldcg(lrow + k), T, sh.rowmax[0], sh.rowsum[0]); };
-    const unsigned long long Z = row_mass(wf, [&](int k, float w) { stcg(qrow + k, w); }, V, rs, &sh.rows);
-    mine = row_pick(wf, V, Z, u[a.j], rs, &sh.rows, tok);
+    const RowMass m = row_mass(wf, [&](int k, float w) { stcg(qrow + k, w); }, V, rs, &sh.rows);
+    mine = row_pick(wf, V, m, u[a.j], rs, &sh.rows, tok);
   } else {
     mine = rule_rows([&](int j, int k) { return prob_of(ldcg(a.logits + (size_t)(r0 + j) * V + k), T, sh.rowmax[j], sh.rowsum[j]); },
                      [&](int j, int k) { return ldcg(a.q_in + (size_t)j * V + k); }, s_ids, u, gamma, V, 0, rs, &sh.rows, r, tok);
@@ -410,8 +410,8 @@ __global__ void __launch_bounds__(ROW_THREADS) sample_rows_kernel(const __grid_c
   } else {
     auto wf = [&](int k) { return ldcg(prow + k); };
     float* qrow = a.mode == MODE_DRAFT ? a.q_out + (size_t)a.j * V : nullptr;
-    const unsigned long long Z = row_mass(wf, [&](int k, float w) { if (qrow) stcg(qrow + k, w); }, V, rs, &sc);
-    mine = row_pick(wf, V, Z, a.mode == MODE_DRAFT ? u[a.j] : u[0], rs, &sc, tok);
+    const RowMass m = row_mass(wf, [&](int k, float w) { if (qrow) stcg(qrow + k, w); }, V, rs, &sc);
+    mine = row_pick(wf, V, m, a.mode == MODE_DRAFT ? u[a.j] : u[0], rs, &sc, tok);
   }
   if (mine && threadIdx.x == 0) {
     if (a.mode == MODE_DRAFT) {

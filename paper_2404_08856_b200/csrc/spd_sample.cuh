@@ -33,26 +33,24 @@ __device__ __forceinline__ bool accept_test(float u, float p, float q) {
 // The sampling kernels give a vocabulary row to a cluster of C CTAs of up to ROW_THREADS threads (C = 1 is
 // an ordinary CTA; any whole number of warps works): CTA `rank` owns the contiguous slice [rank * VC, (rank + 1) * VC), a warp a contiguous
 // piece of it, and the CTAs exchange their integer totals through each other's shared memory, one
-// cluster barrier per draw.  One CTA of 256 threads needs 22 us for a draw from 32000 weights (its
-// latency: every pass is 125 dependent loads deep), the grid-wide form in two launches 8 + 7 us.
+// cluster barrier per draw (about 1 us with the launch of the cluster; one CTA spares it).  Bound by latency: the
+// ids, the two values of every test, the row, the search, one after the other, and few instructions to fetch: a search
+// unrolled over 16 steps of 32 entries took 3200 cycles of a draw from 1000 weights, narrowing 32-fold at a time 900.
+// Device time of the rule alone, 6 rows, us: 1000 entries 5.1 -> 3.5 (all rows accepted, greedy: 6.0 -> 5.1), 32000 entries
+// 7.8 -> 5.1 (10.2 -> 9.4); by one CTA of 256 threads and a serial walk: 3.4 (8.8) and 14 to 26 (25).
 constexpr int ROW_THREADS = 1024, ROW_WARPS = ROW_THREADS / 32, ROW_CTAS_MAX = 8;
 __device__ __forceinline__ int row_warps() { return (int)(blockDim.x >> 5); }
 constexpr int ARG_ROWS = 8;     // rows whose arg-max is taken together
 
 struct RowScratch {
   unsigned long long wsum[ROW_WARPS];
-  float wmax[ROW_WARPS];
-  int widx[ROW_WARPS];
   unsigned long long tot[ROW_CTAS_MAX];            // every CTA's mass
-  float cmax[ROW_CTAS_MAX];                        // its largest weight
-  int cidx[ROW_CTAS_MAX];
-  float amax[ARG_ROWS][ROW_WARPS];                 // arg-max of several rows at once
+  unsigned amax[ARG_ROWS][ROW_WARPS];                 // arg-max of several rows at once
   int aidx[ARG_ROWS][ROW_WARPS];
-  float gmax[ARG_ROWS][ROW_CTAS_MAX];
+  unsigned gmax[ARG_ROWS][ROW_CTAS_MAX];
   int gidx[ARG_ROWS][ROW_CTAS_MAX];
   int arg[ARG_ROWS];
   int result;
-  int first_reject;
 };
 
 struct RowSlice {
@@ -84,128 +82,176 @@ __device__ __forceinline__ void row_piece(const RowSlice& rs, int V, int warp, i
 
 constexpr int ROW_UNROLL = 8;    // loads in flight per thread
 
-// Masses of the row's weights; emit(k, w) sees every weight of this CTA's slice once.  Returns the row's
-// total mass (the same in every CTA); the weights can then be drawn from with row_pick.
+__device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {   // three 32-bit sums of 27-bit parts
+  return (unsigned long long)__reduce_add_sync(0xffffffffu, (unsigned)(v & 0x7ffffffull)) +
+         ((unsigned long long)__reduce_add_sync(0xffffffffu, (unsigned)((v >> 27) & 0x7ffffffull)) << 27) +
+         ((unsigned long long)__reduce_add_sync(0xffffffffu, (unsigned)(v >> 54)) << 54);
+}
+
+// What a row's draws need: the row's total mass (the same in every CTA) and, of this CTA's warps, the mass
+// of warp `lane` and of all up to it.
+struct RowMass {
+  unsigned long long Z, own, upto;
+};
+
+// Masses of the row's weights; emit(k, w) sees every weight of this CTA's slice once.  The weights can then be
+// drawn from with row_pick.  (A second call needs a barrier between them: the scratch is written again.)
 template <class WF, class EM>
-__device__ unsigned long long row_mass(WF wf, EM emit, int V, const RowSlice& rs, RowScratch* sc) {
+__device__ RowMass row_mass(WF wf, EM emit, int V, const RowSlice& rs, RowScratch* sc) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   int k0, k1;
   row_piece(rs, V, warp, k0, k1);
   unsigned long long s = 0;
-  float bm = -1.0f;
-  int bi = 0x7fffffff;
   for (int kb = k0; kb < k1; kb += 32 * ROW_UNROLL) {
     float w[ROW_UNROLL];
 #pragma unroll
     for (int i = 0; i < ROW_UNROLL; ++i) {
       const int k = kb + i * 32 + lane;
-      w[i] = k < k1 ? wf(k) : -1.0f;
+      w[i] = k < k1 ? wf(k) : 0.f;
     }
 #pragma unroll
     for (int i = 0; i < ROW_UNROLL; ++i) {
       const int k = kb + i * 32 + lane;
       if (k < k1) {
         s += to_fixed(w[i]);
-        if (w[i] > bm) { bm = w[i]; bi = k; }
         emit(k, w[i]);
       }
     }
   }
-#pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    s += __shfl_xor_sync(0xffffffffu, s, o);
-    const float om = __shfl_xor_sync(0xffffffffu, bm, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-    if (om > bm || (om == bm && oi < bi)) { bm = om; bi = oi; }
-  }
-  if (lane == 0) { sc->wsum[warp] = s; sc->wmax[warp] = bm; sc->widx[warp] = bi; }
+  s = warp_sum(s);
+  if (lane == 0) sc->wsum[warp] = s;
   __syncthreads();
-  if (warp == 0) {
-    const bool on = lane < row_warps();
-    s = on ? sc->wsum[lane] : 0ull; bm = on ? sc->wmax[lane] : -1.0f; bi = on ? sc->widx[lane] : 0x7fffffff;
+  RowMass m;
+  m.own = m.upto = lane < row_warps() ? sc->wsum[lane] : 0ull;
 #pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      s += __shfl_xor_sync(0xffffffffu, s, o);
-      const float om = __shfl_xor_sync(0xffffffffu, bm, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (om > bm || (om == bm && oi < bi)) { bm = om; bi = oi; }
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long t = __shfl_up_sync(0xffffffffu, m.upto, o);
+    if (lane >= o) m.upto += t;
+  }
+  m.Z = __shfl_sync(0xffffffffu, m.upto, 31);
+  if (rs.C > 1) {
+    if (warp == 0 && lane < rs.C) store_in_cta(&sc->tot[rs.rank], lane, m.Z);
+    cluster_sync_all_threads();
+    m.Z = 0;
+    for (int c = 0; c < rs.C; ++c) m.Z += sc->tot[c];
+  }
+  return m;
+}
+
+// Arg-max (lowest index on ties) of n <= ARG_ROWS rows at once: f(j, k) = value k of row j; the results are
+// left in sc->arg of every CTA.  A warp takes a piece of one row, so that all rows' loads travel together: 6 x 32000 on
+// a cluster of 8 in 7.5 us, 9.5 with the rows one after the other and all warps on each.
+template <class F>
+__device__ void rows_argmax(F f, int n, int V, const RowSlice& rs, RowScratch* sc) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = row_warps();
+  const int VC = (V + rs.C - 1) / rs.C, s0 = min(V, rs.rank * VC), s1 = min(V, s0 + VC);
+  const int P = n < nw ? nw / n : 1, VP = (((s1 - s0 + P - 1) / P) + 31) & ~31;
+  // a value as an unsigned number of the same order (-0 as 0, a NaN below everything)
+  auto key = [](float v) {
+    const unsigned b = __float_as_uint(v + 0.0f);
+    return v != v ? 0u : (b & 0x80000000u ? ~b : b | 0x80000000u);
+  };
+  // largest value of the warp, lowest index on ties (0x7fffffff: no entry)
+  auto reduce = [&](unsigned& bk, int& bi) {
+    const unsigned top = __reduce_max_sync(0xffffffffu, bk);
+    bi = (int)__reduce_min_sync(0xffffffffu, bk == top ? (unsigned)bi : 0x7fffffffu);
+    bk = top;
+  };
+  for (int item = warp; item < n * P; item += nw) {
+    const int j = item / P, pc = item - j * P, k0 = min(s1, s0 + pc * VP), k1 = min(s1, k0 + VP);
+    float bm = -INFINITY;
+    int bi = 0x7fffffff;
+    for (int kb = k0; kb < k1; kb += 32 * ROW_UNROLL) {
+      float w[ROW_UNROLL];
+#pragma unroll
+      for (int i = 0; i < ROW_UNROLL; ++i) {
+        const int k = kb + i * 32 + lane;
+        w[i] = k < k1 ? f(j, k) : -INFINITY;
+      }
+#pragma unroll
+      for (int i = 0; i < ROW_UNROLL; ++i) {
+        const int k = kb + i * 32 + lane;
+        if (k < k1 && (w[i] > bm || bi == 0x7fffffff)) { bm = w[i]; bi = k; }
+      }
     }
-    if (lane < rs.C) {
-      store_in_cta(&sc->tot[rs.rank], lane, s);
-      store_in_cta(&sc->cmax[rs.rank], lane, bm);
-      store_in_cta(&sc->cidx[rs.rank], lane, bi);
+    unsigned bk = bi == 0x7fffffff ? 0u : key(bm);
+    reduce(bk, bi);
+    if (lane == 0) { sc->amax[j][pc] = bk; sc->aidx[j][pc] = bi; }
+  }
+  __syncthreads();
+  for (int j = warp; j < n; j += nw) {
+    unsigned bk = lane < P ? sc->amax[j][lane] : 0u;
+    int bi = lane < P ? sc->aidx[j][lane] : 0x7fffffff;
+    reduce(bk, bi);
+    if (rs.C == 1) {
+      if (lane == 0) sc->arg[j] = bi;
+    } else if (lane < rs.C) {
+      store_in_cta(&sc->gmax[j][rs.rank], lane, bk);
+      store_in_cta(&sc->gidx[j][rs.rank], lane, bi);
     }
   }
-  cluster_sync_all_threads();
-  unsigned long long Z = 0;
-  for (int c = 0; c < rs.C; ++c) Z += sc->tot[c];
-  return Z;
+  if (rs.C > 1) {
+    cluster_sync_all_threads();
+    if (tid < n) {
+      unsigned bk = sc->gmax[tid][0];
+      int bi = sc->gidx[tid][0];
+      for (int c = 1; c < rs.C; ++c) {      // (slices in order: the first of equals has the lowest index)
+        const unsigned ok = sc->gmax[tid][c];
+        const int oi = sc->gidx[tid][c];
+        if (oi != 0x7fffffff && (bi == 0x7fffffff || ok > bk)) { bk = ok; bi = oi; }
+      }
+      sc->arg[tid] = bi;
+    }
+  }
+  __syncthreads();
 }
 
 // The token that uniform u draws from the weights of the preceding row_mass.  Exactly one CTA of the
 // cluster, the one whose slice holds the token, returns true.
 template <class WF>
-__device__ bool row_pick(WF wf, int V, unsigned long long Z, float u, const RowSlice& rs, RowScratch* sc, int& tok) {
+__device__ bool row_pick(WF wf, int V, const RowMass& m, float u, const RowSlice& rs, RowScratch* sc, int& tok) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (Z == 0) {      // no mass at all: the largest weight, lowest index on ties
-    float m = sc->cmax[0];
-    tok = sc->cidx[0];
-    for (int c = 1; c < rs.C; ++c)
-      if (sc->cmax[c] > m) { m = sc->cmax[c]; tok = sc->cidx[c]; }
-    if (tok >= V) tok = 0;      // a row of NaN has no largest weight
+  if (m.Z == 0) {      // no mass at all: the largest weight, lowest index on ties; entries that are no numbers last
+    rows_argmax([&](int, int k) { const float w = wf(k); return w > -1.0f ? w : -1.0f; }, 1, V, rs, sc);
+    tok = sc->arg[0];
+    cluster_sync_all_threads();   // (the exchange buffers may be used again)
     return rs.rank == 0;
   }
-  const unsigned long long T = threshold(Z, u);
+  const unsigned long long T = threshold(m.Z, u);
   unsigned long long base = 0;
-  int cc = 0;
-  while (cc < rs.C - 1 && T >= base + sc->tot[cc]) base += sc->tot[cc++];
-  if (cc != rs.rank) return false;
-  // the warp whose piece the running total crosses T in
-  const unsigned long long own = lane < row_warps() ? sc->wsum[lane] : 0ull;
-  unsigned long long inc = own;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned long long t = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += t;
+  if (rs.C > 1) {
+    int cc = 0;
+    while (cc < rs.C - 1 && T >= base + sc->tot[cc]) base += sc->tot[cc++];
+    if (cc != rs.rank) return false;
   }
-  const unsigned over = __ballot_sync(0xffffffffu, T < base + inc);
+  // the warp whose piece the running total crosses T in
+  const unsigned over = __ballot_sync(0xffffffffu, T < base + m.upto);
   const int ww = over ? __ffs(over) - 1 : row_warps() - 1;
-  base += __shfl_sync(0xffffffffu, inc - own, ww);
+  base += __shfl_sync(0xffffffffu, m.upto - m.own, ww);
   if (warp == ww) {
+    // narrowed 32-fold at a time: a lane sums a run of entries, the lane whose run the total crosses T in is next
     int k0, k1;
     row_piece(rs, V, warp, k0, k1);
-    int found = max(k1 - 1, 0);
-    constexpr int B = 16;          // 32-wide steps looked at together
-    bool hit = false;
-    for (int kb = k0; kb < k1 && !hit; kb += 32 * B) {
-      unsigned long long m[B];
+    int len = k1 - k0;
+    while (true) {
+      const int run = (len + 31) >> 5, b0 = min(k1, k0 + lane * run), b1 = min(min(k1, k0 + len), b0 + run);
+      unsigned long long own = 0;
+#pragma unroll 4
+      for (int k = b0; k < b1; ++k) own += to_fixed(wf(k));
+      unsigned long long upto = own;
 #pragma unroll
-      for (int i = 0; i < B; ++i) {
-        const int k = kb + i * 32 + lane;
-        m[i] = k < k1 ? to_fixed(wf(k)) : 0ull;
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long t = __shfl_up_sync(0xffffffffu, upto, o);
+        if (lane >= o) upto += t;
       }
-#pragma unroll
-      for (int i = 0; i < B; ++i) {
-        if (hit) continue;
-        // the step's total: three 32-bit sums of 27-bit parts
-        const unsigned long long tot = (unsigned long long)__reduce_add_sync(0xffffffffu, (unsigned)(m[i] & 0x7ffffffull)) +
-                                       ((unsigned long long)__reduce_add_sync(0xffffffffu, (unsigned)((m[i] >> 27) & 0x7ffffffull)) << 27) +
-                                       ((unsigned long long)__reduce_add_sync(0xffffffffu, (unsigned)(m[i] >> 54)) << 54);
-        if (T < base + tot) {
-          unsigned long long pre = m[i];
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long t = __shfl_up_sync(0xffffffffu, pre, o);
-            if (lane >= o) pre += t;
-          }
-          const unsigned mask = __ballot_sync(0xffffffffu, base + pre > T);
-          found = kb + i * 32 + __ffs(mask) - 1;
-          hit = true;
-        } else {
-          base += tot;
-        }
-      }
+      const unsigned past = __ballot_sync(0xffffffffu, T < base + upto && b0 < b1);
+      const int l = past ? __ffs(past) - 1 : 0;
+      base += __shfl_sync(0xffffffffu, upto - own, l);
+      k0 += l * run;
+      if (run <= 1) break;
+      len = min(len - l * run, run);
     }
+    const int found = max(min(k0, k1 - 1), 0);
     if (lane == 0) sc->result = found;
   }
   __syncthreads();
@@ -217,65 +263,8 @@ __device__ bool row_pick(WF wf, int V, unsigned long long Z, float u, const RowS
 // One draw.
 template <class WF>
 __device__ bool row_sample(WF wf, int V, float u, const RowSlice& rs, RowScratch* sc, int& tok) {
-  const unsigned long long Z = row_mass(wf, [](int, float) {}, V, rs, sc);
-  return row_pick(wf, V, Z, u, rs, sc, tok);
-}
-
-// Arg-max (lowest index on ties) of n <= ARG_ROWS rows at once: f(j, k) = value k of row j; the results are
-// left in sc->arg of every CTA.
-template <class F>
-__device__ void rows_argmax(F f, int n, int V, const RowSlice& rs, RowScratch* sc) {
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int VC = (V + rs.C - 1) / rs.C, s0 = min(V, rs.rank * VC), s1 = min(V, s0 + VC);
-  for (int j = 0; j < n; ++j) {
-    float bm = -INFINITY;
-    int bi = 0x7fffffff;
-    for (int kb = s0; kb < s1; kb += (int)blockDim.x * 4) {
-      float w[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int k = kb + i * (int)blockDim.x + tid;
-        w[i] = k < s1 ? f(j, k) : -INFINITY;
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int k = kb + i * (int)blockDim.x + tid;
-        if (k < s1 && (w[i] > bm || bi == 0x7fffffff)) { bm = w[i]; bi = k; }
-      }
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      const float om = __shfl_xor_sync(0xffffffffu, bm, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (oi != 0x7fffffff && (bi == 0x7fffffff || om > bm || (om == bm && oi < bi))) { bm = om; bi = oi; }
-    }
-    if (lane == 0) { sc->amax[j][warp] = bm; sc->aidx[j][warp] = bi; }
-  }
-  __syncthreads();
-  for (int j = warp; j < n; j += row_warps()) {
-    const bool on = lane < row_warps();
-    float bm = on ? sc->amax[j][lane] : -INFINITY;
-    int bi = on ? sc->aidx[j][lane] : 0x7fffffff;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      const float om = __shfl_xor_sync(0xffffffffu, bm, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (oi != 0x7fffffff && (bi == 0x7fffffff || om > bm || (om == bm && oi < bi))) { bm = om; bi = oi; }
-    }
-    if (lane < rs.C) { store_in_cta(&sc->gmax[j][rs.rank], lane, bm); store_in_cta(&sc->gidx[j][rs.rank], lane, bi); }
-  }
-  cluster_sync_all_threads();
-  if (tid < n) {
-    float bm = sc->gmax[tid][0];
-    int bi = sc->gidx[tid][0];
-    for (int c = 1; c < rs.C; ++c) {
-      const float om = sc->gmax[tid][c];
-      const int oi = sc->gidx[tid][c];
-      if (oi != 0x7fffffff && (bi == 0x7fffffff || om > bm || (om == bm && oi < bi))) { bm = om; bi = oi; }
-    }
-    sc->arg[tid] = bi;
-  }
-  __syncthreads();
+  const RowMass m = row_mass(wf, [](int, float) {}, V, rs, sc);
+  return row_pick(wf, V, m, u, rs, sc, tok);
 }
 
 // The rejection rule (Sec. 2.1) for one sequence on a cluster: pv(j, k) / qv(j, k) = value k of the target's /
@@ -285,8 +274,9 @@ template <class PV, class QV>
 __device__ bool rule_rows(PV pv, QV qv, const int* ids, const float* ub, int gamma, int V, int greedy, const RowSlice& rs,
                           RowScratch* sc, int& r, int& tok) {
   if (greedy) {
-    for (int j0 = 0;; j0 += ARG_ROWS) {
-      const int n = min(ARG_ROWS, gamma + 1 - j0);
+    // the first row alone, then the others together: a draft that is off mostly is so at once, 4.1 us instead of
+    // 7.5 at 32000 entries (9.4 instead of 7.8 where all of six rows are accepted)
+    for (int j0 = 0, n = 1;; j0 += n, n = min(ARG_ROWS, gamma + 1 - j0)) {
       rows_argmax([&](int j, int k) { return pv(j0 + j, k); }, n, V, rs, sc);
       for (int j = 0; j < n; ++j) {
         r = j0 + j;
@@ -296,12 +286,13 @@ __device__ bool rule_rows(PV pv, QV qv, const int* ids, const float* ub, int gam
       cluster_sync_all_threads();   // the exchange buffers are written again
     }
   }
-  if (threadIdx.x == 0) sc->first_reject = gamma;
-  __syncthreads();
-  for (int j = threadIdx.x; j < gamma; j += blockDim.x)   // the accept tests are independent
-    if (!accept_test(ub[j], pv(j, ids[j]), qv(j, ids[j]))) atomicMin(&sc->first_reject, j);
-  __syncthreads();
-  r = sc->first_reject;
+  // the accept tests are independent; every warp makes all of them, which spares two barriers
+  r = gamma;
+  for (int j0 = 0; j0 < gamma && r == gamma; j0 += 32) {
+    const int j = j0 + (threadIdx.x & 31);
+    const unsigned rej = __ballot_sync(0xffffffffu, j < gamma && !accept_test(ub[j], pv(j, ids[j]), qv(j, ids[j])));
+    if (rej) r = j0 + __ffs(rej) - 1;
+  }
   const int rr = r;
   if (rr < gamma) return row_sample([&](int k) { return fmaxf(0.0f, __fsub_rn(pv(rr, k), qv(rr, k))); }, V, ub[gamma], rs, sc, tok);
   return row_sample([&](int k) { return pv(rr, k); }, V, ub[gamma], rs, sc, tok);
@@ -321,8 +312,8 @@ reject_sample_kernel(const float* __restrict__ p, const float* __restrict__ q, c
   const float* ub = u ? u + (size_t)b * (gamma + 1) : nullptr;
   // a draft id outside [0, V) cannot index a row: the sequence is reported as n_acc = next = -1
   bool bad = false;
-  for (int j = 0; j < gamma; ++j) bad |= (unsigned)idb[j] >= (unsigned)V;
-  if (bad) {      // the same in every CTA of the cluster
+  for (int j = threadIdx.x & 31; j < gamma; j += 32) bad |= (unsigned)idb[j] >= (unsigned)V;
+  if (__any_sync(0xffffffffu, bad)) {      // the same in every CTA of the cluster
     if (rs.rank == 0 && threadIdx.x == 0) { n_acc[b] = -1; next[b] = -1; }
     return;
   }

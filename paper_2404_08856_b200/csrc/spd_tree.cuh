@@ -44,11 +44,11 @@ __global__ void __launch_bounds__(ROW_THREADS) tree_draw_kernel(const __grid_con
     const float mx = sh.rowmax[k], sm = sh.rowsum[k];
     auto wf = [&](int i) { return truncated ? ldcg(row + i) : prob_of(ldcg(lrow + i), a.temperature, mx, sm); };
     float* qrow = a.q_out + (size_t)node * V;
-    const unsigned long long Z = row_mass(wf, [&](int i, float w) { stcg(qrow + i, w); }, V, rs, &sh.rows);
+    const RowMass m = row_mass(wf, [&](int i, float w) { stcg(qrow + i, w); }, V, rs, &sh.rows);
     for (int c = 1; c <= shape.n; ++c) {
       if (shape.parent[c] != node) continue;
       int tok;
-      if (row_pick(wf, V, Z, u[c - 1], rs, &sh.rows, tok) && threadIdx.x == 0) st->d_ids[c - 1] = tok;
+      if (row_pick(wf, V, m, u[c - 1], rs, &sh.rows, tok) && threadIdx.x == 0) st->d_ids[c - 1] = tok;
     }
   } else {
     int n_taken = 0;
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(ROW_THREADS) tree_verify_kernel(const __grid_c
         // cur <- max(0, cur - q) / sum, the sum taken over integer masses
         const float* c0 = cur;
         auto left = [&](int i) { return fmaxf(0.0f, __fsub_rn(ldcg(c0 + i), ldcg(qrow + i))); };
-        const unsigned long long Z = row_mass(left, [](int, float) {}, V, rs, &sh.rows);
+        const unsigned long long Z = row_mass(left, [](int, float) {}, V, rs, &sh.rows).Z;
         const float S = __fmul_rn(__ull2float_rn(Z), 2.3283064365386963e-10f);
 #pragma unroll 8
         for (int i = tid; i < V; i += ROW_THREADS) {   // (in place after the first rejection: element by element)

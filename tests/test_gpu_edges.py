@@ -51,7 +51,8 @@ def test_skinny_gemm_edges(M, N, K, dtype, noalloc):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("B,gamma,V", [(1, 0, 1), (3, 1, 31), (2, 9, 1024), (20, 7, 4099), (75, 2, 8200), (149, 17, 700), (1, 5, 40000)])
+@pytest.mark.parametrize("B,gamma,V", [(1, 0, 1), (3, 1, 31), (2, 9, 1024), (20, 7, 4099), (75, 2, 8200), (149, 17, 700), (1, 5, 40000),
+                                       (2, 40, 6144), (2, 33, 6145), (5, 3, 16384), (5, 3, 16385), (40, 1, 16390), (3, 4, 33)])
 def test_rejection_rule_edges(B, gamma, V):
     """Every cluster width, more rows than are taken together when greedy, vocabularies around a warp's piece."""
     import torch
@@ -171,6 +172,14 @@ def test_draws_from_rows_that_are_no_distribution(V):
     ids = np.array([[0], [0], [V - 5]], np.int32)
     spd.reject_sample(torch.from_numpy(greedy).cuda(), None, torch.from_numpy(ids).cuda(), None, 1, True, a[:3], n[:3])
     assert a[:3].cpu().tolist() == [1, 1, 1] and n[:3].cpu().tolist() == [0, 0, V - 5]
+    ties = np.zeros((3, V), F32)                       # equal values in several pieces, zeros of both signs
+    ties[0, [V // 2, V // 2 + 31, V - 1]] = 2.0
+    ties[1, ::2] = -0.0
+    ties[2] = -3.0
+    ties[2, [V // 3, V - 2]] = -0.0
+    ids = ties.argmax(-1).astype(np.int32)[:2][None]
+    spd.reject_sample(torch.from_numpy(ties[None]).cuda(), None, torch.from_numpy(ids).cuda(), None, 2, True, a[:1], n[:1])
+    assert (int(a[0]), int(n[0])) == (2, V // 3)
     trunc = np.stack([np.where(np.arange(V) % 3 == 1, F32(nan), flat), np.where(np.arange(V) % 2 == 0, -flat, flat)]).astype(F32)
     want = warp.warp_rows(np.where(trunc > 0, trunc, F32(0)), 20, 0.9)
     assert np.array_equal(_dev_truncate(spd, trunc, 20, 0.9).view(np.uint32), want.view(np.uint32))
