@@ -509,16 +509,20 @@ int device_sms(int dev) {
 constexpr size_t TRUNC_ROOM = 6296;      // shared memory kept free of the row (with 256 bins the kernel declares 3 KB)
 bool trunc_fits(int V, int smem_optin) { return (size_t)V * sizeof(float) + TRUNC_ROOM <= (size_t)smem_optin; }
 cudaError_t launch_truncate(const float* in, float* out, int rows, int V, int top_k, float top_p, int smem_optin, cudaStream_t stream) {
-  static int attr[MAX_DEV][2];
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess || dev < 0 || dev >= MAX_DEV) return e != cudaSuccess ? e : cudaErrorInvalidDevice;
   const int smem = V * (int)sizeof(float);
+  static std::atomic<bool> sized[MAX_DEV][2];
   auto go = [&](auto kernel, int slot) {
-    if (attr[dev][slot] < smem) {
-      const cudaError_t r = cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (!sized[dev][slot].load(std::memory_order_acquire)) {
+      // all the kernel may ever have: the limit is shared by every caller of the process, whatever its V
+      cudaFuncAttributes fa{};
+      cudaError_t r = cudaFuncGetAttributes(&fa, (const void*)kernel);
+      if (r == cudaSuccess)
+        r = cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin - (int)fa.sharedSizeBytes);
       if (r != cudaSuccess) return r;
-      attr[dev][slot] = smem;
+      sized[dev][slot].store(true, std::memory_order_release);
     }
     kernel<<<rows, TRUNC_THREADS, smem, stream>>>(in, out, V, top_k, top_p);
     return cudaGetLastError();

@@ -305,3 +305,42 @@ def test_draft_logits_of_every_step_are_kept(dtype):
             assert e.value.status == spd.SPD_EINVAL
         assert np.array_equal(gpu.get_draft_logits(left).view(np.uint32), rows[:left].view(np.uint32))
     gpu.close()
+
+
+@pytest.mark.gpu
+def test_threads_that_truncate_rows_of_different_lengths_at_once():
+    """The kernels' limit on shared memory belongs to the process: no thread may lower it under another's launch.
+    A fresh process, so that the first calls of all threads come together."""
+    import subprocess
+    import sys
+    code = """
+import sys, threading
+import numpy as np, torch
+import paper_2404_08856_b200 as spd
+spd.lib(); torch.cuda.init()
+sizes = [56500, 53000, 40000, 30000, 20000, 13000, 5000, 54500]
+rows = [torch.full((2, V), 1.0 / V, device="cuda") for V in sizes]
+outs = [torch.empty_like(r) for r in rows]
+torch.cuda.synchronize()
+gate, bad = threading.Barrier(len(sizes)), []
+def work(i):
+    torch.cuda.set_device(0)
+    gate.wait()
+    for _ in range(50):
+        try:
+            spd.truncate_probs(rows[i], outs[i], 3, 1.0)
+        except Exception as e:
+            bad.append((sizes[i], str(e)))
+threads = [threading.Thread(target=work, args=(i,)) for i in range(len(sizes))]
+[t.start() for t in threads]; [t.join() for t in threads]
+torch.cuda.synchronize()
+assert not bad, bad[:3]
+for V, o in zip(sizes, outs):
+    assert (o.cpu().numpy() > 0).sum(1).tolist() == [3, 3] and float(o[0, 0]) > 0, V
+print("threads ok")
+"""
+    import os
+    _lib()
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=root, timeout=200)
+    assert r.returncode == 0 and "threads ok" in r.stdout, r.stderr[-2000:]
