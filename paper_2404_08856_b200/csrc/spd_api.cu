@@ -1063,7 +1063,10 @@ spd_status spd_create(const spd_weights* target_w, const spd_weights* draft_w, c
   size_t stage_elems = 0;
   for (const spd_model_cfg* c : {&cfg->target, &cfg->draft}) {
     const size_t e = c->dtype ? 2 : 4;
-    const size_t big = (size_t)(c->vocab > c->d_ffn ? c->vocab : c->d_ffn) * c->d_model * e;
+    size_t rows = c->vocab > c->d_ffn ? c->vocab : c->d_ffn;   // the longer side of the largest matrix
+    if (c->d_model > (int)rows) rows = c->d_model;
+    if (c == &cfg->draft && cfg->draft_adapter_in > (int)rows) rows = cfg->draft_adapter_in;
+    const size_t big = rows * c->d_model * e;
     if (big > stage_elems) stage_elems = big;
   }
   (void)esz_t; (void)esz_d;

@@ -344,3 +344,13 @@ print("threads ok")
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=root, timeout=200)
     assert r.returncode == 0 and "threads ok" in r.stdout, r.stderr[-2000:]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype,tol", [("fp32", 2e-4), ("bf16", 2e-2)])
+def test_models_wider_than_their_vocabulary_and_ffn(dtype, tol):
+    """The largest matrix of the target is d_model x d_model, that of the draft its adapter."""
+    t = synth.ModelCfg(1, 512, 4, 264, 400, False, dtype=dtype)
+    d = synth.ModelCfg(1, 128, 2, 136, 400, False, dtype=dtype)
+    wl = synth.Workload("wide", t, d, 8, 16, 4, 16, adapter_in=512)
+    assert lockstep(wl, False, 1.0, 2, tol, std=0.08)["blocks"] == 2
