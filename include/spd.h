@@ -350,9 +350,11 @@ spd_status spd_reject_sample(const float* p, const float* q, const int32_t* ids,
 spd_status spd_truncate_probs(const float* probs, float* out, int rows, int V, int top_k,
                               float top_p, void* stream);
 
-/* Y[M,N] = X[M,K] W[N,K]^T with the weight-streaming kernel of the verify projections
- * (Eq. 1's linear maps at M = gamma+1 rows).  x, y fp32 DEVICE, w DEVICE in `dtype`;
- * 1 <= M <= 8, K a multiple of 8.  Asynchronous on stream. */
+/* Y[M,N] = X[M,K] W[N,K]^T: the linear maps of Eq. 1 at M = gamma+1 rows, alone.  x, y fp32 DEVICE, w
+ * DEVICE in `dtype`, all 16-byte aligned; 1 <= M <= 8, K a multiple of 8.  Asynchronous on stream.
+ * Where the activations fit a CTA's shared memory (bf16: K <= 6144; fp32: M x K rounded up to a multiple
+ * of 128 <= 49152) the weights are read as they are, once; beyond that they are first repacked into a
+ * growing device buffer and run through the forward kernel's projection. */
 spd_status spd_skinny_gemm(const float* x, const void* w, int dtype, int M, int N, int K,
                            float* y, void* stream);
 
@@ -383,24 +385,24 @@ spd_status spd_wait_selftest(spd_ctx* ctx, int which, unsigned polls);
  * engine or framework that hands out fixed arenas and forbids side allocations), inside
  * a latency-critical loop where the implicit device synchronisation of cudaMalloc/cudaFree
  * is unacceptable, or in a process whose memory budget was fixed at start-up.
- * spd_skinny_gemm keeps a growing device buffer for the repacked weights and allocates
- * it on demand; this variant instead uses a fixed scratch array compiled into the library
+ * spd_skinny_gemm keeps a status block and, for the shapes it repacks, a growing device buffer, both
+ * allocated on demand; this variant instead uses a fixed scratch array compiled into the library
  * (SPD_NOALLOC_MAX_PACKED_BYTES plus a 512-byte header).  Every GPU that loads the library
  * holds that array until the process exits, whether or not this function is ever called.
  *
  *   - x, w, y, dtype, M, N, K, stream: exactly as spd_skinny_gemm (the caller still owns
  *     inputs and outputs).
- *   - Limit: the repacked weights, ceil(N/4)*4 * ceil(K*esz/512)*512 bytes with esz = 2
- *     (bf16) or 4 (fp32), must not exceed SPD_NOALLOC_MAX_PACKED_BYTES; otherwise the call
- *     does nothing, prints one line to stderr and returns SPD_EOVERFLOW.
+ *   - Limit: ceil(N/4)*4 * ceil(K*esz/512)*512 bytes with esz = 2 (bf16) or 4 (fp32), the size of the
+ *     repacked weights, must not exceed SPD_NOALLOC_MAX_PACKED_BYTES; otherwise the call does nothing,
+ *     prints one line to stderr and returns SPD_EOVERFLOW.  The limit is the same for the shapes that
+ *     are not repacked, so that it depends on N, K and dtype alone.
  *   - It calls no cudaMalloc, cudaFree or other allocating routine.
  *   - The first call on each device (with that device current) looks up the device address
  *     of the scratch array and the device properties; make that first call before starting
  *     any stream capture.
- *   - All calls share the one array.  Its contents persist between calls; the words that
- *     must start at zero are cleared on the stream at the start of every call.  Two calls
- *     whose GPU work overlaps (different streams, or different host threads) race on it:
- *     serialise them.
+ *   - All calls share the one array.  Its contents persist between calls; the status word is cleared on
+ *     the stream at the start of every call.  Two calls whose GPU work overlaps (different streams, or
+ *     different host threads) race on it: serialise them.
  * Asynchronous on stream. */
 #define SPD_NOALLOC_MAX_PACKED_BYTES (16u << 20)
 spd_status spd_skinny_gemm_noalloc(const float* x, const void* w, int dtype, int M, int N,

@@ -891,7 +891,7 @@ spd_status launch_prefill_attn(spd_ctx* ctx, const __nv_bfloat16* kc, const __nv
 }
 
 // Dense forward of rows X [R][d] (fp32, device; positions 0..R-1) through every layer of a
-// bf16 model: fills the KV cache rows 0..R-1 and leaves the final residual stream in X.  Seven launches
+// bf16 model: fills the KV cache rows 0..R-1 and leaves the final residual stream in X.  Eight launches
 // a layer; a projection whose reader can add K slices up is sliced where that fills the device.  `rows`: those
 // of the call's larger pass, which the buffers are sized for.
 spd_status prefill_tc(spd_ctx* ctx, ModelHost& mh, float* X, int R, int rows) {
@@ -928,7 +928,7 @@ spd_status prefill_tc(spd_ctx* ctx, ModelHost& mh, float* X, int R, int rows) {
   return SPD_OK;
 }
 
-// Buffers of a context that are not part of a model: device state, barrier pool, uniforms,
+// Buffers of a context that are not part of a model: device state, grid barrier, uniforms,
 // draft distributions, prefill staging, output ids, pinned state copy, events, graph stream.
 spd_status alloc_ctx_buffers(spd_ctx* ctx) {
   const spd_cfg* cfg = &ctx->cfg;
@@ -966,8 +966,8 @@ bool use_tc_prefill(const ModelHost& mh) { return mh.cfg.dtype == 1; }
 
 // ------------------------------------------------------------------------------ fixed scratch
 // Scratch of spd_skinny_gemm_noalloc: lives in the library image, so no allocation call is
-// ever made for it.  Layout: [0,256) grid-barrier word, [256,512) kernel status block,
-// [512, ...) the streaming-layout copy of the weight matrix.
+// ever made for it.  Layout: [0,256) unused, [256,512) kernel status block, [512, ...) the streaming-layout
+// copy of the weight matrix (shapes whose activations do not fit shared memory).
 constexpr size_t NOALLOC_HEADER = 512;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_HEADER + SPD_NOALLOC_MAX_PACKED_BYTES];
 
@@ -1570,7 +1570,7 @@ struct spd_batch {
   int drafted_gamma = -1;
   int last_rows = 0;
   std::vector<void*> allocs;
-  // One step (forward + probability rows + sampling / rule kernels) is a fixed sequence of ~10 small
+  // One step (forward + probability rows + sampling / rule kernels) is a fixed sequence of eight
   // launches per layer whose arguments never change (lengths and tokens live on the device), so it
   // is captured once as a CUDA graph per (model, rows per sequence, draft step) and replayed.
   cudaStream_t cap_stream = nullptr;
@@ -1757,7 +1757,7 @@ spd_status spd_batch_create(spd_ctx* const* seqs, int B, spd_batch** out) {
   if (!ctx) return SPD_EINVAL;
   const int gm = ctx->cfg.gamma_max > 0 ? ctx->cfg.gamma_max : 1;
   if (B * (gm + 1) > BATCH_ROWS_MAX || B * 2 > BATCH_ROWS_MAX)
-    return fail(ctx, SPD_EINVAL, "batch x (gamma_max + 1) rows must fit one 128-row tile");
+    return fail(ctx, SPD_EINVAL, "batch x (gamma_max + 1) rows must not exceed 128");
   if (ctx->cfg.target.dtype != 1 || ctx->cfg.draft.dtype != 1)
     return fail(ctx, SPD_EINVAL, "the batched path needs bf16 models (tensor-core GEMMs)");
   const spd_ctx* origin0 = ctx->origin ? ctx->origin : ctx;

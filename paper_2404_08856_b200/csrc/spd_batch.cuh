@@ -2,7 +2,7 @@
 // step: the method's premise is that a target call is bound by streaming the parameters, Sec. 1 and
 // Sec. 4 "Metrics", so B sequences should share that stream).  The rows of all sequences --
 // B x (gamma + 1) for a verify step, B x 2 for a draft step -- go through each projection as one
-// dense GEMM on the tcgen05 tensor cores (spd_prefill.cuh); attention, rotary embedding, cache
+// dense GEMM on the tcgen05 tensor cores (spd_gemm.cuh); attention, rotary embedding, cache
 // append, the rejection rule and the commit stay per sequence: every sequence has its own cache,
 // its own length and its own accepted count (Sec. 2.1's rule is stated per sequence).
 #pragma once
@@ -16,7 +16,7 @@ struct BatchSeq {
   int pos_base_t, pos_base_d;   // rows in front of the text in the target's / draft's cache
 };
 
-constexpr int BATCH_ROWS_MAX = 128;   // one 128-row tile of the tensor-core GEMM
+constexpr int BATCH_ROWS_MAX = 128;   // rows of a batched step: what its buffers are sized for
 
 // Row (b, m) of a batched launch.  Verify: m = 0 the pending token, m >= 1 draft token m-1, cache row
 // and rotary position origin_b + m.  Draft step j: the two rows [token before, token to extend] at

@@ -201,3 +201,47 @@ def test_batch_argument_errors_and_mixing_with_single_calls():
         assert got[k][:n] == want[k][:n]
     bt.close()
     b.close(); a.close(); other.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("B,gamma,d_model,heads", [
+    (40, 1, 2048, 32),      # 1280 (sequence, head) units on 1184 warps: some take a second one
+    (64, 1, 2048, 32),      # ... and the most rows a batch may have
+    (16, 7, 256, 4),        # 128 rows, eight per sequence: no padded query row, heads of 64
+    (16, 7, 256, 2)])       # heads of 128
+def test_batches_at_the_limits_against_the_same_sequences_alone(B, gamma, d_model, heads):
+    """Caches of 1, 2 and 3 key / value tiles and around them.  Logits of a batched verify step against spd_verify of
+    each sequence on its own behind the same cache (two paths of the same precision: the bound of the small bf16
+    models); the third round replays captured launches after a prefill that has outgrown the scratch they were
+    captured with."""
+    spd = _lib()
+    t = synth.ModelCfg(1, d_model, heads, 264, 1024, False, dtype="bf16")
+    d = synth.ModelCfg(1, 128, 2, 344, 1024, False, dtype="bf16")
+    wl = synth.Workload("limits", t, d, 0, 16, gamma, 16)
+    tw, dw = H.build_weights(wl, 0.1)
+    lead = H.make_gpu(wl, tw, dw, 300, 1.0, True, gamma_max=gamma)
+    seqs = [lead] + [lead.fork() for _ in range(B - 1)]
+    tile = 32 if d_model // heads == 64 else 16
+    g = np.random.default_rng(B)
+    lengths = [max(1, (1 + k % 3) * tile - gamma + (-2, -1, 0, 1, 5)[k % 5]) for k in range(B)]
+    prompts = [g.integers(0, 1024, n).astype(np.int32) for n in lengths]
+    bt, M = spd.SpdBatch(seqs), gamma + 1
+    for step in range(3):
+        if step == 2:
+            lead.prefill(None, g.integers(0, 1024, 280).astype(np.int32))
+        at = [(len(p), int(p[-1]), c.prefill(None, p)) for c, p in zip(seqs, prompts)]
+        ids = bt.draft(gamma)
+        acc, nxt = bt.verify(gamma)
+        rows = bt.get_logits(B * M).reshape(B, M, -1)
+        for k, c in enumerate(seqs):
+            c.rollback(*at[k])
+            a, n = c.verify(gamma, None, draft_ids=ids[k])
+            alone = c.get_logits(M)
+            assert np.abs(rows[k] - alone).max() < 2e-2, (step, k)
+            top = np.sort(alone, axis=1)[:, -2:]
+            if (top[:, 1] - top[:, 0]).min() > 4e-2:
+                assert (a, n) == (int(acc[k]), int(nxt[k])), (step, k)
+    bt.close()
+    for c in seqs[1:]:
+        c.close()
+    lead.close()

@@ -3,9 +3,9 @@
 spd_skinny_gemm_noalloc is meant for hosts where this library may not call cudaMalloc or
 cudaFree: programs whose device memory belongs to another allocator, latency-critical
 loops that cannot afford the device-wide synchronisation an allocation implies, processes
-with a memory budget fixed at start-up.  It keeps its scratch (barrier word, status block,
-repacked weights) in a fixed array inside the library, shared by all calls.  This test calls
-it several times in a row with different shapes and data -- each call sees whatever the one
+with a memory budget fixed at start-up.  It keeps its scratch (status block, repacked weights of the
+shapes that are repacked) in a fixed array inside the library, shared by all calls.  This test calls
+it several times in a row with different shapes and data -- a call that repacks sees whatever the one
 before left in the scratch -- and compares each result with spd_skinny_gemm on the same inputs
 and with an fp64 matrix product, checks that a warmed call leaves the amount of free device
 memory exactly as it found it, that its status word reads clean afterwards, and that a matrix
@@ -33,7 +33,9 @@ def _lib():
 def test_noalloc_gemm_matches_regular_entry_point_twice_in_a_row():
     import torch
     spd = _lib()
-    cases = [(6, 1000, 4096, 1), (3, 260, 688, 0), (8, 1536, 2048, 1)]   # the last reuses a dirty scratch
+    # the first three run on the weights as they are; the others (activations beyond a CTA's shared memory) repack
+    # into the scratch array, each over what the one before left there
+    cases = [(6, 1000, 4096, 1), (3, 260, 688, 0), (8, 1536, 2048, 1), (6, 1000, 6400, 1), (8, 500, 6272, 0), (3, 333, 6152, 1)]
     for idx, (M, N, K, dtype) in enumerate(cases):
         g = np.random.default_rng(100 + idx)
         x = g.standard_normal((M, K)).astype(F32)
