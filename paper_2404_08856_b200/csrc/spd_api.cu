@@ -482,15 +482,41 @@ cudaError_t launch_rows(void (*kernel)(KA...), int rows, int C, int threads, cud
   return cudaLaunchKernelEx(&cfg, kernel, KA(args)...);
 }
 
-// CTAs per row.  Below ~6000 entries one: a cluster's launch and barrier cost more than its share of the row is worth.  Then
-// 4 and 8 (the portable cluster size), as long as all rows are on the device at once.  Device time of the rule on one /
-// 16 sequences, us, with 1, 4, 8 CTAs of 512 threads: 4000 entries 4.2, 5.0, 4.9 / 4.3, 5.2, 5.7; 6000 4.1, 4.8, 5.0 / 5.0, 5.3, 5.6;
-// 8000 5.5, 4.9, 5.0 / 5.7, 5.2, 6.2; 16000 8.9, 5.4, 5.1 / 9.2, 5.6, 6.1; 32000 8.1, 5.7, 5.1 / 13.4, 7.0, 5.9.  (2 CTAs are never the
-// best: 5.3 at 8000.)
-int row_ctas(int n_sm, int rows, int V) {
-  int C = V <= 6144 ? 1 : (V <= 16384 ? 4 : ROW_CTAS_MAX);
-  while (C > 1 && rows * C > n_sm) C >>= 1;
+// CTAs per row of a draw.  Below ~6000 entries one: a cluster's launch and barrier cost more than its share of the row is
+// worth.  Then 4 and 8 (the portable cluster size) as long as all rows are on the device at once; clusters of 8 CTAs that have
+// an SM each leave part of every GPC unused, so that 16 of them take two waves (draws from 16 rows of 32000: 10.4 us, 6.7 with 4 CTAs).
+// Device time of the rule on 1 / 8 / 32 sequences, rows not in L2, us, with 1, 4, 8 CTAs of 512 threads: 4000 entries 4.1, 4.9,
+// 4.7 / 5.5, 5.5, 5.3 / 5.8, 5.7, -; 8000 5.2, 4.9, 5.0 / 7.6, 5.7, 5.6 / 7.5, 5.9, -; 16000 8.1, 5.2, 5.1 / 12.8, 7.1, 6.1 / 15.4, 8.0, -;
+// 32000 15.9, 8.0, 6.3 / 19.9, 9.8, 7.3 / 26.8, 11.7, -.
+int row_ctas(int n_sm, int rows, int V, int threads = ROW_THREADS) {
+  int C = V <= 6144 ? 1 : (V <= 12288 ? 4 : ROW_CTAS_MAX);
+  while (C > 1 && rows * C > (C == ROW_CTAS_MAX && threads > ROW_THREADS / 2 ? n_sm / 2 : n_sm)) C >>= 1;
   return C;
+}
+
+// Launch of the rule alone on B sequences: CTAs per sequence and threads per CTA (few per entry: with a small vocabulary many
+// sequences share an SM).
+struct RuleLaunch { int C, threads; };
+RuleLaunch rule_launch(int n_sm, int B, int V, int greedy) {
+  RuleLaunch l{row_ctas(n_sm, B, V, ROW_THREADS / 2), 0};
+  int slice = (V + l.C - 1) / l.C, most, per = 4;
+  if (!greedy) {
+    // 32 sequences of 32000 on 4 CTAs: 512 threads 11.7, 1024 threads 9.2 us; of 16000: 8.0 and 7.6 (in L2: 5.8 and 6.5)
+    most = slice > 6144 ? ROW_THREADS : ROW_THREADS / 2;
+  } else {
+    // Up to gamma + 1 rows a sequence, so clusters pay from shorter rows on.  First token rejected / most accepted, us: few
+    // sequences, 4000 entries on 1 / 8 CTAs 2.9 / 6.8 and 3.8 / 6.4, 8000 3.5 / 11.8 and 3.8 / 7.3; many (8), 2000 entries on 1 / 4 CTAs
+    // 7.2 / 7.5 and 5.2 / 5.7, 4000 on 4 / 8 6.6 / 7.0 and 5.4 / 5.8; 8 CTAs of 512 / 1024 threads, 16000 entries 9.2 / 9.6 and 7.6 / 8.1
+    const bool many = B >= RULE_MANY;
+    l.C = many ? (V < 2000 ? 1 : (V < 4000 ? 4 : ROW_CTAS_MAX)) : (V <= 4096 ? 1 : ROW_CTAS_MAX);
+    while (l.C > 1 && B * l.C > (l.C == ROW_CTAS_MAX ? n_sm / 2 : n_sm)) l.C >>= 1;
+    slice = (V + l.C - 1) / l.C;
+    most = slice > 1500 && (many || (l.C > 1 && slice > 2000)) ? ROW_THREADS : ROW_THREADS / 2;
+    per = 2;
+  }
+  l.threads = ((slice + per - 1) / per + 31) / 32 * 32;
+  if (l.threads > most) l.threads = most;
+  return l;
 }
 
 // SMs of a device, asked for once.
@@ -2104,15 +2130,8 @@ spd_status spd_reject_sample(const float* p, const float* q, const int32_t* ids,
   if (cudaGetDevice(&dev) != cudaSuccess) return SPD_ECUDA;
   const int n_sm = device_sms(dev);
   if (n_sm < 1) return SPD_ECUDA;
-  // four entries of a slice per thread up to 512 threads (with a small vocabulary many sequences share an SM), more than
-  // 512 only for slices of over 8000 entries: 32000 entries on 1 / 2 / 4 / 8 CTAs, 32 (8: 4) sequences, us: 512 threads 13.6 / 10.5 /
-  // 7.2 / 5.7, 1024 threads 10.9 / 8.3 / 6.8 / 6.7
-  // (greedy decoding mostly looks at more rows than one: clusters are worth it from shorter rows on, 6 accepted rows of 6000 on
-  // 1 / 4 CTAs 8.5 / 7.2 us, of 16000 on 4 / 8 CTAs 9.1 / 7.6)
-  const int C = row_ctas(n_sm, B, greedy ? V + V / 2 : V), slice = (V + C - 1) / C, most = slice > 8000 ? ROW_THREADS : ROW_THREADS / 2;
-  int threads = ((slice + 3) / 4 + 31) / 32 * 32;
-  if (threads > most) threads = most;
-  return launch_rows(reject_sample_kernel, B, C, threads, static_cast<cudaStream_t>(stream), false, p, q, ids, u, gamma, V, greedy, C, n_acc,
+  const RuleLaunch l = rule_launch(n_sm, B, V, greedy);
+  return launch_rows(reject_sample_kernel, B, l.C, l.threads, static_cast<cudaStream_t>(stream), false, p, q, ids, u, gamma, V, greedy, l.C, n_acc,
                      next) == cudaSuccess ? SPD_OK : SPD_ECUDA;
 }
 

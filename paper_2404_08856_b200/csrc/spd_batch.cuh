@@ -408,7 +408,7 @@ __global__ void __launch_bounds__(ROW_THREADS) batch_verify_kernel(const BatchSe
   };
   auto qv = [&](int j, int k) { return ldcg(q_all + ((size_t)b * gamma + j) * V + k); };
   int r, tok;
-  const bool mine = rule_rows(pv, qv, s_ids, u ? u + row0 : nullptr, gamma, V, greedy, rs, &sc, r, tok);
+  const bool mine = rule_rows(pv, qv, s_ids, u ? u + row0 : nullptr, gamma, V, greedy, rs, &sc, gridDim.x / C, r, tok);
   if (mine && threadIdx.x == 0) {
     st->n_acc = r;
     st->next = tok;

@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(ROW_THREADS) sample_step_kernel(const __grid_c
     mine = row_pick(wf, V, m, u[a.j], rs, &sh.rows, tok);
   } else {
     mine = rule_rows([&](int j, int k) { return prob_of(ldcg(a.logits + (size_t)(r0 + j) * V + k), T, sh.rowmax[j], sh.rowsum[j]); },
-                     [&](int j, int k) { return ldcg(a.q_in + (size_t)j * V + k); }, s_ids, u, gamma, V, 0, rs, &sh.rows, r, tok);
+                     [&](int j, int k) { return ldcg(a.q_in + (size_t)j * V + k); }, s_ids, u, gamma, V, 0, rs, &sh.rows, 1, r, tok);
   }
   if (mine && threadIdx.x == 0) {
     if (a.mode == MODE_DRAFT) {
@@ -406,7 +406,7 @@ __global__ void __launch_bounds__(ROW_THREADS) sample_rows_kernel(const __grid_c
     }
     __syncthreads();
     mine = rule_rows([&](int j, int k) { return ldcg(prow + (size_t)j * V + k); },
-                     [&](int j, int k) { return ldcg(a.q_in + (size_t)j * V + k); }, s_ids, u, a.gamma, V, 0, rs, &sc, r, tok);
+                     [&](int j, int k) { return ldcg(a.q_in + (size_t)j * V + k); }, s_ids, u, a.gamma, V, 0, rs, &sc, 1, r, tok);
   } else {
     auto wf = [&](int k) { return ldcg(prow + k); };
     float* qrow = a.mode == MODE_DRAFT ? a.q_out + (size_t)a.j * V : nullptr;

@@ -36,11 +36,12 @@ __device__ __forceinline__ bool accept_test(float u, float p, float q) {
 // cluster barrier per draw (about 1 us with the launch of the cluster; one CTA spares it).  Bound by latency: the
 // ids, the two values of every test, the row, the search, one after the other, and few instructions to fetch: a search
 // unrolled over 16 steps of 32 entries took 3200 cycles of a draw from 1000 weights, narrowing 32-fold at a time 900.
-// Device time of the rule alone, 6 rows, us: 1000 entries 5.1 -> 3.5 (all rows accepted, greedy: 6.0 -> 5.1), 32000 entries
-// 7.8 -> 5.1 (10.2 -> 9.4); by one CTA of 256 threads and a serial walk: 3.4 (8.8) and 14 to 26 (25).
+// Device time of the rule on one sequence, 6 rows not in L2, sampled, us: 1000 entries 3.5 (with clusters, a barrier more and the
+// unrolled search 5.4; one CTA of 256 threads and a serial walk 4.0), 32000 entries 6.4 (8.4; 28).
 constexpr int ROW_THREADS = 1024, ROW_WARPS = ROW_THREADS / 32, ROW_CTAS_MAX = 8;
 __device__ __forceinline__ int row_warps() { return (int)(blockDim.x >> 5); }
 constexpr int ARG_ROWS = 8;     // rows whose arg-max is taken together
+constexpr int RULE_MANY = 8;    // sequences from which on a greedy rule takes all its rows at once
 
 struct RowScratch {
   unsigned long long wsum[ROW_WARPS];
@@ -269,14 +270,17 @@ __device__ bool row_sample(WF wf, int V, float u, const RowSlice& rs, RowScratch
 
 // The rejection rule (Sec. 2.1) for one sequence on a cluster: pv(j, k) / qv(j, k) = value k of the target's /
 // draft's row j (qv unused when greedy), ids [gamma] draft ids (each already known to lie in [0, V)), ub
-// [gamma+1] uniforms.  Exactly one CTA returns true, with the accepted count r and the next token.
+// [gamma+1] uniforms; `rows`: the sequences of the launch.  Exactly one CTA returns true, with the accepted count r
+// and the next token.
 template <class PV, class QV>
 __device__ bool rule_rows(PV pv, QV qv, const int* ids, const float* ub, int gamma, int V, int greedy, const RowSlice& rs,
-                          RowScratch* sc, int& r, int& tok) {
+                          RowScratch* sc, int rows, int& r, int& tok) {
   if (greedy) {
-    // the first row alone, then the others together: a draft that is off mostly is so at once, 4.1 us instead of
-    // 7.5 at 32000 entries (9.4 instead of 7.8 where all of six rows are accepted)
-    for (int j0 = 0, n = 1;; j0 += n, n = min(ARG_ROWS, gamma + 1 - j0)) {
+    // Few sequences: the first row alone, then the others together, as a draft that is off mostly is so at once.  One sequence,
+    // 32000 entries on 8 CTAs, first token rejected / most accepted, us: 4.7 / 11.8, all rows together 9.4 / 9.7, row by row on one
+    // CTA 6.2 / 53.  Of many sequences one gets further nearly always, and the launch lasts as long as the longest: together
+    // (32 sequences 14.5 instead of 16.9).
+    for (int j0 = 0, n = rows < RULE_MANY ? 1 : min(ARG_ROWS, gamma + 1);; j0 += n, n = min(ARG_ROWS, gamma + 1 - j0)) {
       rows_argmax([&](int j, int k) { return pv(j0 + j, k); }, n, V, rs, sc);
       for (int j = 0; j < n; ++j) {
         r = j0 + j;
@@ -319,7 +323,7 @@ reject_sample_kernel(const float* __restrict__ p, const float* __restrict__ q, c
   }
   int r, tok;
   const bool mine = rule_rows([&](int j, int k) { return pb[(size_t)j * V + k]; }, [&](int j, int k) { return qb[(size_t)j * V + k]; },
-                              idb, ub, gamma, V, greedy, rs, &sc, r, tok);
+                              idb, ub, gamma, V, greedy, rs, &sc, gridDim.x / C, r, tok);
   if (mine && threadIdx.x == 0) { n_acc[b] = r; next[b] = tok; }
 }
 

@@ -52,7 +52,8 @@ def test_skinny_gemm_edges(M, N, K, dtype, noalloc):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("B,gamma,V", [(1, 0, 1), (3, 1, 31), (2, 9, 1024), (20, 7, 4099), (75, 2, 8200), (149, 17, 700), (1, 5, 40000),
-                                       (2, 40, 6144), (2, 33, 6145), (5, 3, 16384), (5, 3, 16385), (40, 1, 16390), (3, 4, 33)])
+                                       (2, 40, 6144), (2, 33, 6145), (5, 3, 16384), (5, 3, 16385), (40, 1, 16390), (3, 4, 33),
+                                       (8, 9, 1999), (8, 7, 4000), (9, 8, 4097), (10, 8, 8000), (18, 1, 16400), (7, 8, 4096)])
 def test_rejection_rule_edges(B, gamma, V):
     """Every cluster width, more rows than are taken together when greedy, vocabularies around a warp's piece."""
     import torch
