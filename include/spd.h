@@ -276,7 +276,8 @@ void spd_batch_destroy(spd_batch* batch);
 /* gamma draft steps for every sequence (Sec. 2.1), each step one pass over the draft's weights.
  *   uniforms   fp32 [B, gamma], host or device; may be NULL when greedy
  *   draft_ids  int32 [B, gamma], out, host or device, may be NULL
- * The draft distributions are kept inside the batch for spd_batch_verify. */
+ * The draft distributions are kept inside the batch for spd_batch_verify.  Batched steps replay graphs of
+ * their own and cannot be captured (SPD_ECUDA). */
 spd_status spd_batch_draft(spd_batch* batch, int gamma, const float* uniforms, int32_t* draft_ids);
 
 /* One target call on the B x (gamma+1) rows [pending_b, x_b1..x_b,gamma], then per sequence the
@@ -308,7 +309,8 @@ spd_status spd_get_draft_logits(spd_ctx* ctx, float* logits, int rows);
 /* Rollback / resynchronisation: declares that the committed text is n_text tokens long
  * (prompt included, pending token excluded), that prev_token is its last token and
  * pending_token the token to feed next.  KV rows of positions >= the new length are
- * treated as stale; rows below it must belong to the same sequence.  O(1). */
+ * treated as stale; rows below it must belong to the same sequence.  O(1).  SPD_ECUDA while the
+ * stream is being captured. */
 spd_status spd_rollback(spd_ctx* ctx, int n_text, int32_t prev_token, int32_t pending_token);
 spd_status spd_get_state(spd_ctx* ctx, int32_t* n_text, int32_t* pending_token);
 
